@@ -491,13 +491,50 @@ int run_launch(cb_plan* p, const Window& win, const double* w, void* const* outs
                      &smem, &per_sm);
     if (rc != CB_OK) return rc;
     if (A.stages < max_nb + 1) return launch_direct();  // too deep for shared memory
-    // Persistent grid. bf16 prediction-only launches with K >= 3 stream faster
-    // over 3/4 of the SMs (one CTA each) than over all of them (measured on
-    // GB300, repeatable within 0.5 %: FLUX 99 -> 103 %, PixArt 96 -> 104 %,
-    // DiT-512 95 -> 101 % of the copy peak). Launches that update hidden states
-    // are bound by their consumers and use every SM.
+    const int stages_all = A.stages;
+    const size_t smem_all = smem;
+    // Bytes in flight. HBM serves a mix of reads and writes best when no more is
+    // asked of it than covers its latency; beyond that reads and writes turn
+    // the bus around more often. GB300, DiT-XL/2 256^2 shapes, every SM, KB in
+    // flight per SM (all that fits -> here): predictions with K = 1 100.0 ->
+    // 83.8 us (48), K = 2 136 -> 120 (64), K = 3 169 -> 151 (120), K = 4 206 ->
+    // 188 (128); full-step epilogue from fp32 features 176 -> 159 (100). The
+    // more is read per byte written, the flatter the optimum and the higher.
+    // Launches that hold a group's stages keep two groups' worth; those with
+    // K >= 2 are bound by their consumers and any depth serves them.
+    if (!grouped || K == 1) {
+        double rd = 0, wr = 0, units = 0;
+        for (int i = 0; i < items; ++i) {
+            const double e = (double)A.numel[i], x = A.resid[i] ? (double)res : 0.0;
+            rd += e * (A.nb[i] * K * (cb16 ? 2.0 : 4.0) + x);
+            units += e * A.nb[i];
+            wr += e * x;
+            for (int m = 0; m < A.nb[i]; ++m)
+                if (A.m_out[A.first[i] + m]) wr += e * (A.out_bf16 ? 2.0 : 4.0);
+        }
+        const double ratio = rd / wr, kb = grouped ? 96 : ratio < 1.25 ? 48 : ratio < 2.5 ? 76 : 120;
+        const double unit = rd / units * te_bulk;
+        const int most = (int)(kb * 1024.0 / unit / per_sm + 0.5);
+        const int least = std::max(grouped ? 2 * max_nb : 2, per_sm == 1 ? 3 : 2);
+        // bf16 features leave the consumers the bound: those keep every stage
+        if (!(grouped && cb16)) {
+            const int keep = std::max(most, least);
+            if (keep < A.stages) {
+                A.stages = keep;
+                smem = cbk::bulk_smem_bytes(A.stage_chunks, A.stage_gate_bytes, keep);
+            }
+        }
+    }
+    // Persistent grid: every SM, except that bf16 prediction-only launches with
+    // K >= 5, whose stages are too large to be limited in number, limit the
+    // SMs instead (FLUX.1-dev, 3/4 of the SMs with all stages 1788 us, all of
+    // them with three stages 1800 us, with all stages 1898 us).
     double frac = 1.0;
-    if (cb16 && !grouped && K >= 3) frac = 0.75;
+    if (cb16 && !grouped && K >= 5 && tiles >= 8LL * p->dev.sms) {
+        frac = 0.75;
+        A.stages = stages_all;
+        smem = smem_all;
+    }
     const long long ctas = std::max(1LL, (long long)((double)p->dev.sms * per_sm * frac));
     const int grid = (int)(tiles < ctas ? tiles : ctas);
     rc = clear_status();
