@@ -30,8 +30,9 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CFLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2"]
-SOURCES = ["extrapolate.cu", "extrapolate_gated.cu", "extrapolate_bulk.cu", "extrapolate_bulk_gated.cu",
-           "push.cu", "epilogue.cu", "static_status.cu", "plan.cpp"]
+SOURCES = ["extrapolate.cu", "extrapolate_gated.cu", "extrapolate_precise.cu", "extrapolate_bulk.cu", "extrapolate_bulk_gated.cu",
+           "extrapolate_bulk_precise.cu", "extrapolate_bulk_precise_fp32.cu", "extrapolate_bulk_strided.cu",
+           "extrapolate_bulk_strided_fp32.cu", "push.cu", "epilogue.cu", "static_status.cu", "plan.cpp"]
 
 
 def _nvcc() -> str:

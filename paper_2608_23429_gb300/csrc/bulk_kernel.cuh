@@ -21,13 +21,15 @@
 //     registers, and guarded elements are recomputed from those registers;
 //   * with hidden states: stages are released after the member's arithmetic,
 //     guarded elements are recomputed from shared memory (so the history
-//     values die early). The producer also stages each tile's bf16 hidden
-//     state (one more chunk with the group's last member) and the consumers
+//     values die early). The producer also stages each tile's hidden state
+//     (behind the chunks of the group's first member) and the consumers
 //     hold the group's member stages until the hidden state is written (the
 //     host guarantees more stages than members, so holding cannot starve the
 //     producer). With gates, each member's stage also carries the gate rows
 //     of the batches its tile touches, so that no consumer waits on a global
 //     load.
+// Launches with fp32 predictions or hidden states (PRECISE) have kernels of
+// their own: see precise_tile.
 // The same kernel runs a full step's epilogue (cb_cache_push_residual) as a
 // one-entry history of weight 1 whose member addresses are the new features;
 // with copy_out the outputs (the ring slot) receive the features converted.
@@ -48,22 +50,26 @@
 namespace cbk {
 namespace {
 
-// Thread map. With one CTA per SM, one 8-element vector per consumer thread
-// and tile: 16 consumer warps for bf16 tiles (512 vectors; 17 warps cap
+// Thread map (bulk_shape). With one CTA per SM, one 8-element vector per consumer
+// thread and tile: 16 consumer warps for bf16 tiles (512 vectors; 17 warps cap
 // registers at 96), 8 for fp32 tiles (256 vectors). Launches that carry few
-// bytes per unit (most K = 1 launches, and bf16 launches with small K: see
-// bulk_ctas_per_sm) pay the consumers' fixed cost per unit more often; they run two CTAs of 8
+// bytes per unit (most K = 1 launches, and bf16 launches with small K) pay the
+// consumers' fixed cost per unit more often; they run two CTAs of 8
 // consumer warps per SM (two independent pipelines), bf16 threads taking two
 // vectors per tile. An earlier map of 8 consumer warps with two vectors each
 // on one CTA left the launches with hidden states issue-bound.
-template <bool CB16, int K, bool GROUPED, bool GATED>
+template <bool CB16, int K, bool GROUPED, bool GATED, bool PRECISE>
 struct Shape {
-    static constexpr int ctas_per_sm = bulk_ctas_per_sm(K, CB16, GROUPED, GATED);
-    static constexpr int consumer_warps = (CB16 && ctas_per_sm == 1) ? 16 : 8;
+    static constexpr BulkShape b = bulk_shape(K, CB16, GROUPED, GATED, PRECISE);
+    static constexpr int ctas_per_sm = b.ctas_per_sm;
+    static constexpr int consumer_warps = b.consumer_warps;
     static constexpr int consumers = consumer_warps * 32;
     static constexpr int threads = consumers + 32;  // plus the producer warp
+    static constexpr int tile = b.tile;             // elements of one unit
+    static constexpr int chunk = tile * (CB16 ? 2 : 4);  // bytes of one history entry's share of a tile
+    static constexpr int vecs = tile / kVecElems / consumers;  // vectors per consumer thread per tile
+    static_assert(vecs * kVecElems * consumers == tile, "a tile's vectors spread evenly over the consumers");
 };
-constexpr int kChunkBytes = 8192;   // one history entry's share of a tile
 constexpr int kBarrierBytes = 256;  // full[S] and empty[S] barriers, S <= kMaxStages
 static_assert(2 * 8 * kMaxStages <= kBarrierBytes, "barrier block holds every stage's barriers");
 // A consumer warp hands one stage back to the producer: every lane fences its
@@ -80,143 +86,359 @@ __device__ __forceinline__ void release_stage(uint32_t empty_bar, int lane) {
     if (lane == 0) mbar_arrive(empty_bar);
 }
 
-// GROUPED: some item updates a hidden state or has several members (stage
-// holding, hidden-state staging); prediction-only launches compile without
-// that bookkeeping. GATED (with GROUPED): the hidden state receives g_b * P_b,
-// with a per-(batch, channel) gate per member.
-// ONE: the full-step epilogue (copy_out with bf16 hidden states or none): a
-// one-entry history of weight 1, whose member step needs no weighted sum
-// (member_one); compiled apart so that each kernel carries only its own path.
-template <int K, bool CB16, bool GROUPED, bool GATED, bool ONE = false>
-__global__ void __launch_bounds__(Shape<CB16, K, GROUPED, GATED>::threads, Shape<CB16, K, GROUPED, GATED>::ctas_per_sm)
-    extrapolate_bulk_kernel(const __grid_constant__ ExtrapArgs A) {
-    static_assert(!ONE || K == 1, "the epilogue is a one-entry history");
-    extern __shared__ __align__(128) unsigned char smem[];
-    constexpr int NCW = Shape<CB16, K, GROUPED, GATED>::consumer_warps;
-    constexpr int NCT = Shape<CB16, K, GROUPED, GATED>::consumers;
-    constexpr long long TE = tile_elems(CB16);  // 8 KB per history chunk for both cache types
+// Bytes of a ragged tile of n elements that are copied: whole 16-byte pieces.
+// The history's tensors are padded to CB_CACHE_ALIGN, so the last piece may
+// reach past the tensor; a full step's new features are not, and what is left
+// of them (less than 16 bytes) is read from global memory.
+template <int ES>
+__device__ __forceinline__ uint32_t ragged_bytes(const ExtrapArgs& A, long long n) {
+    const uint32_t b = (uint32_t)n * ES;
+    return A.copy_out ? b & ~15u : (b + 15u) & ~15u;
+}
+
+// The producer lane: every unit's history chunks, and what travels with them,
+// from global into shared memory, in the consumers' order.
+template <int K, bool CB16, bool GROUPED, bool GATED, bool PRECISE, bool STRIDED>
+__device__ __forceinline__ void produce(const ExtrapArgs& A, uint32_t full0, uint32_t empty0, uint32_t buf0,
+                                        uint32_t stage_bytes) {
+    using Sh = Shape<CB16, K, GROUPED, GATED, PRECISE>;
+    constexpr long long TE = Sh::tile;
     constexpr int ES = CB16 ? 2 : 4;
-    constexpr int NV = (int)(TE / kVecElems);     // vectors per tile: 512 (bf16) or 256 (fp32)
-    constexpr int U = NV >= NCT ? NV / NCT : 1;   // vectors per consumer thread per tile
-    static_assert(NV % NCT == 0 || NCT % NV == 0, "vectors spread evenly over the consumers");
-    static_assert(TE * ES == kChunkBytes, "one tile of one history entry is one chunk");
     const int S = A.stages;
-    const uint32_t full0 = smem_addr(smem);
-    const uint32_t empty0 = full0 + 8u * (uint32_t)S;
-    const uint32_t buf0 = smem_addr(smem + kBarrierBytes);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) {
-            mbar_init(full0 + 8u * s, 1);
-            mbar_init(empty0 + 8u * s, NCW);
+    unsigned u = 0;               // units issued
+    uint32_t ps = 0, wraps = 0;   // stage of the next unit; times the ring has wrapped
+    // one tile of item `it`: a unit per member; false when a wait ran out
+    auto issue = [&](int it, long long e0, bool whole, uint32_t bytes) {
+        const int first = A.first[it];
+        const int nb = GROUPED ? A.nb[it] : 1;
+        const unsigned char* resid = GROUPED ? reinterpret_cast<const unsigned char*>(A.resid[it]) : nullptr;
+        // gate rows b0..b1 of the batches this tile touches (b1 <= b0 + 1:
+        // the host stages gates only when a batch holds a tile or more)
+        uint32_t gbytes = 0;
+        size_t gsrc = 0;
+        if (GATED && A.stage_gate_bytes && resid && whole && A.i_row[it] != 0) {
+            const long long row = A.i_row[it];
+            const long long b0 = e0 / row, b1 = (e0 + TE - 1) / row;
+            const size_t gs = A.gate_bf16 ? 2 : 4;
+            gsrc = (size_t)b0 * A.i_hidden[it] * gs;
+            gbytes = (uint32_t)((b1 - b0 + 1) * A.i_hidden[it] * gs);
         }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-
-    // the stage stays held through the member's arithmetic (see the consumers)
-    constexpr bool LATE = GROUPED || (CB16 && K >= 7);
-    const int C = GROUPED ? A.stage_chunks : K;
-    const uint32_t stage_bytes = (uint32_t)C * kChunkBytes + (GATED ? A.stage_gate_bytes : 0u);
-    if (warp == NCW) {  // ---------------------------------- producer
-        if (lane != 0) return;
-        int it = 0;
-        unsigned u = 0;               // units issued
-        uint32_t ps = 0, wraps = 0;   // stage of the next unit; times the ring has wrapped
-        bool ok = true;
-        for (int tile = blockIdx.x; ok && tile < A.tiles_total; tile += gridDim.x) {
-            while (tile >= A.tile_begin[it + 1]) ++it;
-            const long long numel = A.numel[it];
-            const long long e0 = (long long)(tile - A.tile_begin[it]) * TE;
-            // consumers read shared memory only for whole tiles of aligned items;
-            // for the ragged last tile (or a misaligned item) the stage is
-            // cycled without data and they recompute from global memory
-            const bool full_tile = A.vec_ok[it] && e0 + TE <= numel;
-            const uint32_t bytes = full_tile ? (uint32_t)kChunkBytes : 0u;
-            const int first = A.first[it];
-            const int nb = GROUPED ? A.nb[it] : 1;
-            const unsigned char* resid = GROUPED ? reinterpret_cast<const unsigned char*>(A.resid[it]) : nullptr;
-            // gate rows b0..b1 of the batches this tile touches (b1 <= b0 + 1:
-            // the host stages gates only when a batch holds a tile or more)
-            uint32_t gbytes = 0;
-            size_t gsrc = 0;
-            if (GATED && A.stage_gate_bytes && resid && full_tile && A.i_row[it] != 0) {
-                const long long row = A.i_row[it];
-                const long long b0 = e0 / row, b1 = (e0 + TE - 1) / row;
-                const size_t gs = A.gate_bf16 ? 2 : 4;
-                gsrc = (size_t)b0 * A.i_hidden[it] * gs;
-                gbytes = (uint32_t)((b1 - b0 + 1) * A.i_hidden[it] * gs);
+        for (int m = 0; m < nb; ++m) {
+            const uint32_t stage = ps;
+            if (wraps > 0 && !mbar_wait(empty0 + 8u * stage, (wraps - 1) & 1u, A.wait_ns)) {
+                record(A.status, 2);
+                return false;
             }
-            for (int m = 0; m < nb; ++m) {
-                const uint32_t stage = ps;
-                if (wraps > 0 && !mbar_wait(empty0 + 8u * stage, (wraps - 1) & 1u, A.wait_ns)) {
-                    record(A.status, 2);
-                    ok = false;
-                    break;
-                }
-                ++u;
-                if (++ps == (uint32_t)S) {
-                    ps = 0;
-                    ++wraps;
-                }
-                // the tile's bf16 hidden state travels with its last member
-                const bool with_x = GROUPED && A.stage_x && resid && full_tile && m == nb - 1;
-                const uint32_t xbytes = with_x ? (uint32_t)(TE * 2) : 0u;
-                const uint32_t gb = (GATED && A.m_gate[first + m]) ? gbytes : 0u;
-                mbar_expect_tx(full0 + 8u * stage, (uint32_t)K * bytes + xbytes + gb);
-                if (A.withhold_first && u == 1) continue;
-                const uint32_t dst = buf0 + stage * stage_bytes;
-                if (bytes) {
+            ++u;
+            if (++ps == (uint32_t)S) {
+                ps = 0;
+                ++wraps;
+            }
+            // a whole tile's hidden state travels with its first member
+            const uint32_t xbytes = GROUPED && resid && whole && m == 0 ? A.stage_x_bytes : 0u;
+            const uint32_t gb = (GATED && A.m_gate[first + m]) ? gbytes : 0u;
+            mbar_expect_tx(full0 + 8u * stage, (uint32_t)K * bytes + xbytes + gb);
+            if (A.withhold_first && u == 1) continue;
+            const uint32_t dst = buf0 + stage * stage_bytes;
+            if (bytes) {
 #pragma unroll
-                    for (int j = 0; j < K; ++j)
-                        bulk_g2s(dst + j * (uint32_t)kChunkBytes, hist_ptr(A, j, A.m_off[first + m]) + e0 * ES, bytes,
-                                 full0 + 8u * stage);
-                }
-                if (xbytes) bulk_g2s(dst + K * (uint32_t)kChunkBytes, resid + e0 * 2, xbytes, full0 + 8u * stage);
-                if (gbytes && A.m_gate[first + m])
-                    bulk_g2s(dst + C * (uint32_t)kChunkBytes,
-                             reinterpret_cast<const unsigned char*>(A.m_gate[first + m]) + gsrc, gbytes,
+                for (int j = 0; j < K; ++j)
+                    bulk_g2s(dst + j * (uint32_t)Sh::chunk, hist_ptr(A, j, A.m_off[first + m]) + e0 * ES, bytes,
                              full0 + 8u * stage);
             }
+            if (xbytes)
+                bulk_g2s(dst + K * (uint32_t)Sh::chunk, resid + e0 * (A.resid_bf16 ? 2 : 4), xbytes,
+                         full0 + 8u * stage);
+            if (gb)
+                bulk_g2s(dst + K * (uint32_t)Sh::chunk + A.stage_x_bytes,
+                         reinterpret_cast<const unsigned char*>(A.m_gate[first + m]) + gsrc, gb, full0 + 8u * stage);
         }
-        // never leave while copies into this CTA's shared memory are in flight:
-        // wait for every unit still in the ring; after one wait runs out (a unit
-        // whose copies were never issued) the others get the short limit
-        unsigned long long drain_ns = A.wait_ns > kMinDrainNs ? A.wait_ns : kMinDrainNs;
-        bool drained = true;
-        for (unsigned q = u > (unsigned)S ? u - S : 0; q < u; ++q)
-            if (!mbar_wait(full0 + 8u * (q % S), (q / S) & 1u, drain_ns)) {
-                drained = false;
-                drain_ns = kMinDrainNs;
-            }
-        if (!drained) record(A.status, 4);
-        return;
-    }
-
-    // ------------------------------------------------------------ consumers
-    const int c = threadIdx.x;
-    const unsigned char* stages = smem + kBarrierBytes;
-    auto chunk = [&](uint32_t stage, int j) { return stages + stage * stage_bytes + (size_t)j * kChunkBytes; };
-    auto gate_stage = [&](uint32_t stage) -> const void* { return stages + stage * stage_bytes + (size_t)C * kChunkBytes; };
-    int it = 0;
-    uint32_t cs = 0, cph = 0;  // stage of the next unit to consume and its phase parity
-    for (int tile = blockIdx.x; tile < A.tiles_total; tile += gridDim.x) {
+        return true;
+    };
+    int it = 0, tile = blockIdx.x;
+    bool ok = true;
+    for (; ok && tile < A.tiles_total; tile += gridDim.x) {
         while (tile >= A.tile_begin[it + 1]) ++it;
-        const long long numel = A.numel[it];
+        const long long e0 = (long long)(tile - A.tile_begin[it]) * TE;
+        const bool whole = !STRIDED || e0 + TE <= A.numel[it];
+        ok = issue(it, e0, whole, whole ? (uint32_t)Sh::chunk : ragged_bytes<ES>(A, A.numel[it] - e0));
+    }
+#pragma unroll 1
+    for (; ok && tile < A.tiles_total + A.n_ragged; tile += gridDim.x) {
+        it = A.ragged[tile - A.tiles_total];
+        const long long e0 = (long long)(A.tile_begin[it + 1] - A.tile_begin[it]) * TE;
+        ok = issue(it, e0, false, ragged_bytes<ES>(A, A.numel[it] - e0));
+    }
+    // never leave while copies into this CTA's shared memory are in flight:
+    // wait for every unit still in the ring; after one wait runs out (a unit
+    // whose copies were never issued) the others get the short limit
+    unsigned long long drain_ns = A.wait_ns > kMinDrainNs ? A.wait_ns : kMinDrainNs;
+    bool drained = true;
+    for (unsigned q = u > (unsigned)S ? u - S : 0; q < u; ++q)
+        if (!mbar_wait(full0 + 8u * (q % S), (q / S) & 1u, drain_ns)) {
+            drained = false;
+            drain_ns = kMinDrainNs;
+        }
+    if (!drained) record(A.status, 4);
+}
+
+// Elements i, i + 1 of a ragged tile (n elements, of which the first `staged`
+// lie in the chunk at p) as words of a vector; zero past the end.
+// TAIL: some elements may not be staged (a full step's new features).
+template <bool CB16, bool TAIL>
+__device__ __forceinline__ uint2 ragged_pair(const unsigned char* p, int i, int n, int staged,
+                                             const unsigned char* global) {
+    uint2 w = make_uint2(0u, 0u);
+    if (i >= n) return w;
+    if (!TAIL || i + 1 < staged) {
+        if constexpr (CB16)
+            w.x = *reinterpret_cast<const uint32_t*>(p + 2 * i);
+        else
+            w = *reinterpret_cast<const uint2*>(p + 4 * i);
+    } else if constexpr (CB16) {
+        const uint16_t* q = reinterpret_cast<const uint16_t*>(global) + i;
+        w.x = q[0] | (i + 1 < n ? (uint32_t)q[1] << 16 : 0u);
+    } else {
+        const uint32_t* q = reinterpret_cast<const uint32_t*>(global) + i;
+        w = make_uint2(q[0], i + 1 < n ? q[1] : 0u);
+    }
+    return w;
+}
+
+// The consumers of launches with fp32 predictions or hidden states: every
+// element takes the compensated sum (sum_vec), so nothing is recomputed and
+// each stage goes back to the producer as soon as its values, and the hidden
+// state behind the first member's, are in registers. The arithmetic (five
+// packed or scalar FMA-pipe operations per history value and element) bounds
+// these launches, not HBM alone.
+//
+// A thread holds vecs vectors of eight elements. In a whole tile they are
+// contiguous; in the ragged last tile of a tensor they are four pairs each,
+// adjacent threads on adjacent pairs, so that any length is covered from
+// shared memory with the same arithmetic (and bits).
+//
+// precise_tile: one tile of one item. RAGGED: any length n <= tile, pairs as
+// above. False when a wait ran out.
+struct Cursor {
+    uint32_t stage = 0, phase = 0;  // of the next unit to consume
+};
+template <typename Sh, int K, bool CB16, bool GROUPED, bool GATED, bool RAGGED>
+__device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long long e0, int n, Cursor& cur,
+                                             uint32_t full0, uint32_t empty0, const unsigned char* stages,
+                                             uint32_t stage_bytes, int lane) {
+    constexpr int ES = CB16 ? 2 : 4;
+    constexpr int NCT = Sh::consumers;
+    constexpr int U = Sh::vecs;
+    const int c = threadIdx.x;
+    const int nb = GROUPED ? A.nb[it] : 1;
+    const int first = A.first[it];
+    void* resid = GROUPED ? A.resid[it] : nullptr;
+    // gates wait in registers through the sums, unless those need the registers
+    // (DiT-XL/2 512^2, K = 8: 785 against 825 us; K = 4: 596 against 589)
+    constexpr bool LATE_GATES = GATED && !RAGGED && K >= 6;
+    const int held = RAGGED ? (int)ragged_bytes<ES>(A, n) / ES : 0;  // elements in the chunks
+    // first element of vector v of this thread, and of pair q of its vector v
+    auto at = [&](int v) { return (v * NCT + c) * kVecElems; };
+    auto pair_at = [&](int v, int q) { return 2 * (c + NCT * (4 * v + q)); };
+    auto put = [&](void* p, bool bf16, int v, const uint32_t (&o)[8]) {
+        if constexpr (!RAGGED) {
+            store_o8(p, bf16, e0 + at(v), o);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                store_o2(p, bf16, e0 + pair_at(v, q), n - pair_at(v, q), bf16 ? o[q] : o[2 * q], o[2 * q + 1]);
+        }
+    };
+    const bool gated = GATED && resid != nullptr && A.i_row[it] != 0;  // items without a shape carry no gate
+    unsigned gi[U];
+    if constexpr (GATED && !RAGGED) {
+        long long ev[U];
+#pragma unroll
+        for (int v = 0; v < U; ++v) ev[v] = e0 + at(v);
+        if (gated) gate_offsets<U>(A, it, e0, ev, gi);
+    }
+    Acc<U> acc;
+    Finite fin;
+    if (GROUPED && RAGGED && resid != nullptr)  // not staged: asked for before the wait for the stage
+        resid_begin<U>(acc, [&](int v, float (&x)[8]) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = pair_at(v, q);
+                x[2 * q] = i < n ? load_elem(resid, A.resid_bf16, e0 + i) : 0.0f;
+                x[2 * q + 1] = i + 1 < n ? load_elem(resid, A.resid_bf16, e0 + i + 1) : 0.0f;
+            }
+        });
+#pragma unroll 1
+    for (int m = 0; m < nb; ++m) {
+        // gates from global memory, asked for before the wait for the stage
+        float g[U][8];
+        if constexpr (GATED) {
+            const void* gp = gated ? A.m_gate[first + m] : nullptr;
+#pragma unroll
+            for (int v = 0; v < U; ++v) {
+                if (LATE_GATES) continue;
+                if (!RAGGED && gp != nullptr) {
+                    load_x8(gp, A.gate_bf16, (long long)gi[v], g[v]);
+                    continue;
+                }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) g[v][e] = 1.0f;
+                if (RAGGED && gp != nullptr)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int i = pair_at(v, q);
+                        if (i >= n) continue;
+                        unsigned g0, g1;
+                        gate_offset_pair(A, it, e0 + i, g0, g1);
+                        g[v][2 * q] = load_elem(gp, A.gate_bf16, g0);
+                        if (i + 1 < n) g[v][2 * q + 1] = load_elem(gp, A.gate_bf16, g1);
+                    }
+            }
+        }
+        const uint32_t stage = cur.stage;
+        if (!__all_sync(~0u, mbar_wait(full0 + 8u * stage, cur.phase, A.wait_ns))) {
+            if (lane == 0) record(A.status, 1);
+            return false;
+        }
+        if (++cur.stage == (uint32_t)A.stages) {
+            cur.stage = 0;
+            cur.phase ^= 1u;
+        }
+        const unsigned char* base = stages + stage * stage_bytes;
+        RawVecs<K, CB16, U> raw;
+#pragma unroll
+        for (int v = 0; v < U; ++v)
+#pragma unroll
+            for (int j = 0; j < K; ++j) {
+                const unsigned char* chunk = base + j * Sh::chunk;
+                if constexpr (!RAGGED) {
+                    const unsigned char* p = chunk + at(v) * ES;
+                    raw[v][j][0] = *reinterpret_cast<const uint4*>(p);
+                    if constexpr (!CB16) raw[v][j][CB16 ? 0 : 1] = *reinterpret_cast<const uint4*>(p + 16);
+                } else {
+                    const unsigned char* src = hist_ptr(A, j, A.m_off[first + m]) + e0 * ES;
+                    uint2 w[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) w[q] = ragged_pair<CB16, K == 1>(chunk, pair_at(v, q), n, held, src);
+                    if constexpr (CB16) {
+                        raw[v][j][0] = make_uint4(w[0].x, w[1].x, w[2].x, w[3].x);
+                    } else {
+                        raw[v][j][0] = make_uint4(w[0].x, w[0].y, w[1].x, w[1].y);
+                        raw[v][j][CB16 ? 0 : 1] = make_uint4(w[2].x, w[2].y, w[3].x, w[3].y);
+                    }
+                }
+            }
+        if (GROUPED && !RAGGED && m == 0 && resid != nullptr)
+            resid_begin<U>(acc, [&](int v, float (&x)[8]) {
+                if (A.stage_x_bytes)
+                    load_x8(base + K * Sh::chunk, A.resid_bf16, at(v), x);
+                else
+                    load_x8(resid, A.resid_bf16, e0 + at(v), x);
+            });
+        release_stage(empty0 + 8u * stage, lane);
+        void* out = A.m_out[first + m];
+        bool want = out != nullptr;
+        if constexpr (K == 1) {
+            if (want && A.copy_out) {  // a full step: the slot receives the features converted
+#pragma unroll
+                for (int v = 0; v < U; ++v) {
+                    uint32_t o[8];
+                    copy_o8<CB16>(A.out_bf16, raw[v][0], o);
+                    put(out, A.out_bf16, v, o);
+                }
+                want = false;
+            }
+        }
+        member_precise<K, CB16, U, GATED>(
+            A, want, raw, resid != nullptr, acc, fin,
+            [&](int v, float (&gv)[8]) {
+                if constexpr (GATED) {
+                    const void* gp = LATE_GATES && gated ? A.m_gate[first + m] : nullptr;
+                    if (gp != nullptr)
+                        load_x8(gp, A.gate_bf16, (long long)gi[v], gv);
+                    else
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) gv[e] = LATE_GATES ? 1.0f : g[v][e];
+                }
+            },
+            [&](int v, const uint32_t (&o)[8]) { put(out, A.out_bf16, v, o); });
+    }
+    if (resid != nullptr ? !resid_precise<K, U>(A, acc, fin,
+                                                [&](int v, const uint32_t (&o)[8]) { put(resid, A.resid_bf16, v, o); })
+                         : !fin.all()) {
+#pragma unroll 1
+        for (int v = 0; v < U; ++v)
+#pragma unroll 1
+            for (int e = 0; e < kVecElems; ++e) {
+                const int i = RAGGED ? pair_at(v, e >> 1) + (e & 1) : at(v) + e;
+                if (i < n) scalar_element<CB16>(A, K, it, e0 + i);
+            }
+    }
+    return true;
+}
+
+// The ragged last tiles, after every whole tile of the launch: a loop of its
+// own, so that their loads and stores cost the loop over whole tiles neither
+// registers nor instruction cache (inside it they cost 5 to 15 %).
+template <typename Sh, int K, bool CB16, bool GROUPED, bool GATED>
+__device__ __forceinline__ bool ragged_tiles(const ExtrapArgs& A, int tile, Cursor& cur, uint32_t full0,
+                                             uint32_t empty0, const unsigned char* stages, uint32_t stage_bytes,
+                                             int lane) {
+#pragma unroll 1
+    for (; tile < A.tiles_total + A.n_ragged; tile += gridDim.x) {
+        const int it = A.ragged[tile - A.tiles_total];
+        const long long e0 = (long long)(A.tile_begin[it + 1] - A.tile_begin[it]) * Sh::tile;
+        if (!precise_tile<Sh, K, CB16, GROUPED, GATED, true>(A, it, e0, (int)(A.numel[it] - e0), cur, full0, empty0,
+                                                             stages, stage_bytes, lane))
+            return false;
+    }
+    return true;
+}
+
+// Items whose sources are off the 16-byte grid (a full step's new features
+// only): element by element from global memory, without the pipeline.
+template <typename Sh, int K, bool CB16>
+__device__ __forceinline__ void scalar_items(const ExtrapArgs& A) {
+    if (!A.any_scalar) return;
+#pragma unroll 1
+    for (int it = 0; it < A.n_items; ++it) {
+        if (A.vec_ok[it]) continue;
+        const long long numel = A.numel[it], step = (long long)gridDim.x * Sh::consumers;
+#pragma unroll 1
+        for (long long e = (long long)blockIdx.x * Sh::consumers + threadIdx.x; e < numel; e += step)
+            scalar_element<CB16>(A, K, it, e);
+    }
+}
+
+// The consumers of every other launch, over the whole tiles (see the head of
+// this file).
+template <int K, bool CB16, bool GROUPED, bool GATED, bool ONE>
+__device__ __forceinline__ bool fast_tiles(const ExtrapArgs& A, int& tile, Cursor& cur, uint32_t full0,
+                                           uint32_t empty0, const unsigned char* stages, uint32_t stage_bytes,
+                                           uint32_t gates_at, int lane) {
+    using Sh = Shape<CB16, K, GROUPED, GATED, false>;
+    constexpr int NCT = Sh::consumers;
+    constexpr long long TE = Sh::tile;
+    constexpr int ES = CB16 ? 2 : 4;
+    constexpr int U = Sh::vecs;
+    // the stage stays held through the member's arithmetic (see below)
+    constexpr bool LATE = GROUPED || (CB16 && K >= 7);
+    const int c = threadIdx.x;
+    const int S = A.stages;
+    auto chunk = [&](uint32_t stage, int j) { return stages + stage * stage_bytes + (size_t)j * Sh::chunk; };
+    auto gate_stage = [&](uint32_t stage) -> const void* { return stages + stage * stage_bytes + gates_at; };
+    int it = 0;
+    for (; tile < A.tiles_total; tile += gridDim.x) {
+        while (tile >= A.tile_begin[it + 1]) ++it;
         const long long e0 = (long long)(tile - A.tile_begin[it]) * TE;
         const int nb = GROUPED ? A.nb[it] : 1;
         const int first = A.first[it];
         void* resid = GROUPED ? A.resid[it] : nullptr;
-        // whole aligned tiles come from shared memory; the ragged last tile of a
-        // tensor and misaligned items take the compensated scalar path
-        const bool full_tile = A.vec_ok[it] && e0 + TE <= numel;
         // with a hidden state, every member's stage stays held until the hidden
         // state is written, so that its guarded elements can be recomputed
-        const bool hold = GROUPED && full_tile && resid != nullptr;
-        const bool mine = NV >= NCT || c < NV;  // fp32 tiles have fewer vectors than consumers
+        const bool hold = GROUPED && resid != nullptr;
         // stage of member m of this tile (nb < S: one wrap at most)
-        const uint32_t s0 = cs;
+        const uint32_t s0 = cur.stage;
         auto stage_of = [&](int m) { return s0 + m < (uint32_t)S ? s0 + m : s0 + m - (uint32_t)S; };
         long long ev[U];
 #pragma unroll
@@ -231,28 +453,26 @@ __global__ void __launch_bounds__(Shape<CB16, K, GROUPED, GATED>::threads, Shape
         Acc<U> acc;
         acc.zero();
         for (int m = 0; m < nb; ++m) {
-            const uint32_t stage = cs;
+            const uint32_t stage = cur.stage;
             // the give-up is warp-uniform: no lane leaves while its warp-mates
             // go on to a __syncwarp
-            if (!__all_sync(~0u, mbar_wait(full0 + 8u * stage, cph, A.wait_ns))) {
+            if (!__all_sync(~0u, mbar_wait(full0 + 8u * stage, cur.phase, A.wait_ns))) {
                 if (lane == 0) record(A.status, 1);
-                return;
+                return false;
             }
-            if (++cs == (uint32_t)S) {
-                cs = 0;
-                cph ^= 1u;
+            if (++cur.stage == (uint32_t)S) {
+                cur.stage = 0;
+                cur.phase ^= 1u;
             }
             RawVecs<K, CB16, U> raw;
-            if (full_tile && mine) {
 #pragma unroll
-                for (int v = 0; v < U; ++v)
+            for (int v = 0; v < U; ++v)
 #pragma unroll
-                    for (int j = 0; j < K; ++j) {
-                        const unsigned char* p = chunk(stage, j) + (size_t)(ev[v] - e0) * ES;
-                        raw[v][j][0] = *reinterpret_cast<const uint4*>(p);
-                        if constexpr (!CB16) raw[v][j][CB16 ? 0 : 1] = *reinterpret_cast<const uint4*>(p + 16);
-                    }
-            }
+                for (int j = 0; j < K; ++j) {
+                    const unsigned char* p = chunk(stage, j) + (size_t)(ev[v] - e0) * ES;
+                    raw[v][j][0] = *reinterpret_cast<const uint4*>(p);
+                    if constexpr (!CB16) raw[v][j][CB16 ? 0 : 1] = *reinterpret_cast<const uint4*>(p + 16);
+                }
             // gates of this member (staged rows or global memory), read as
             // each vector is accumulated
             const void* gp = GATED ? A.m_gate[first + m] : nullptr;
@@ -270,84 +490,135 @@ __global__ void __launch_bounds__(Shape<CB16, K, GROUPED, GATED>::threads, Shape
             // and recompute from shared memory, which frees the history values'
             // registers early (bf16 K >= 7 would otherwise spill under the cap)
             if (!LATE) release_stage(empty0 + 8u * stage, lane);
-            if (full_tile && mine) {
-                void* out = member_out<K, CB16, U>(A, first + m, ev, raw);
-                if constexpr (ONE) {
-                    if (resid != nullptr) member_one<K, CB16, U, GATED>(raw, acc, gate);
-                } else if (A.precise) {
-                    member_precise<K, CB16, U, GATED>(A, out, ev, raw, resid != nullptr, acc, gate);
-                } else if constexpr (LATE) {
-                    auto exact = [&](int v, int e, float& hi, float& lo) {
-                        const size_t off = (size_t)(ev[v] - e0 + e) * ES;
-                        float p = 0.0f, cc = 0.0f;
+            void* out = member_out<K, CB16, U>(A, first + m, ev, raw);
+            if constexpr (ONE) {
+                if (resid != nullptr) member_one<K, CB16, U, GATED>(raw, acc, gate);
+            } else if constexpr (LATE) {
+                auto exact = [&](int v, int e, float& hi, float& lo) {
+                    const size_t off = (size_t)(ev[v] - e0 + e) * ES;
+                    float p = 0.0f, cc = 0.0f;
 #pragma unroll
-                        for (int j = 0; j < K; ++j) {
-                            const unsigned char* src = chunk(stage, j) + off;
-                            const float f = CB16 ? __uint_as_float((uint32_t)(*reinterpret_cast<const uint16_t*>(src)) << 16)
-                                                 : *reinterpret_cast<const float*>(src);
-                            dot2_step(A.w_hi[j], A.w_lo[j], f, p, cc);
-                        }
-                        two_sum(p, cc, hi, lo);
-                    };
-                    member_fast<K, CB16, U, false, GATED>(A, A.m_off[first + m], out, ev, raw, resid != nullptr,
-                                                          acc, gate, exact);
-                } else {
-                    member_fast<K, CB16, U, true, GATED>(A, A.m_off[first + m], out, ev, raw, resid != nullptr,
-                                                         acc, gate);
-                }
+                    for (int j = 0; j < K; ++j) {
+                        const unsigned char* src = chunk(stage, j) + off;
+                        const float f = CB16 ? __uint_as_float((uint32_t)(*reinterpret_cast<const uint16_t*>(src)) << 16)
+                                             : *reinterpret_cast<const float*>(src);
+                        dot2_step(A.w_hi[j], A.w_lo[j], f, p, cc);
+                    }
+                    two_sum(p, cc, hi, lo);
+                };
+                member_fast<K, CB16, U, false, GATED>(A, A.m_off[first + m], out, ev, raw, resid != nullptr,
+                                                      acc, gate, exact);
+            } else {
+                member_fast<K, CB16, U, true, GATED>(A, A.m_off[first + m], out, ev, raw, resid != nullptr,
+                                                     acc, gate);
             }
             if (LATE && !hold) release_stage(empty0 + 8u * stage, lane);
         }
         if (GROUPED && hold) {
-            const uint32_t last = stage_of(nb - 1);
+            // the bf16 hidden state, behind the first member's chunks
             auto xload = [&](int v, float (&x)[8]) {
-                if (A.stage_x)
-                    unpack_bf16x8(*reinterpret_cast<const uint4*>(chunk(last, K) + (size_t)(ev[v] - e0) * 2), x);
-                else
-                    load_x8(resid, A.resid_bf16, ev[v], x);
+                unpack_bf16x8(*reinterpret_cast<const uint4*>(chunk(s0, K) + (size_t)(ev[v] - e0) * 2), x);
             };
-            if (!mine) {
-            } else if (!ONE && A.precise) {
-                resid_precise<U>(A, ev, acc, resid, xload);
-            } else {
-                // Dot2 of x + sum_b P_b for one element, from the held stages
-                auto exact = [&](int v, int e, float xe, float& hi, float& lo) {
-                    const size_t off = (size_t)(ev[v] - e0 + e) * ES;
-                    float tp = xe, tc = 0.0f;
-                    for (int m = 0; m < nb; ++m) {
-                        const uint32_t st = stage_of(m);
-                        float p = 0.0f, cc = 0.0f, h, l, qq;
+            // Dot2 of x + sum_b P_b for one element, from the held stages
+            auto exact = [&](int v, int e, float xe, float& hi, float& lo) {
+                const size_t off = (size_t)(ev[v] - e0 + e) * ES;
+                float tp = xe, tc = 0.0f;
+                for (int m = 0; m < nb; ++m) {
+                    const uint32_t st = stage_of(m);
+                    float p = 0.0f, cc = 0.0f, h, l, qq;
 #pragma unroll
-                        for (int j = 0; j < K; ++j) {
-                            const unsigned char* src = chunk(st, j) + off;
-                            const float f = CB16 ? __uint_as_float((uint32_t)(*reinterpret_cast<const uint16_t*>(src)) << 16)
-                                                 : *reinterpret_cast<const float*>(src);
-                            dot2_step(A.w_hi[j], A.w_lo[j], f, p, cc);
-                        }
-                        two_sum(p, cc, h, l);
-                        // a member without a gate adds like an ungated one (as exact_resid)
-                        const void* gm = GATED ? A.m_gate[first + m] : nullptr;
-                        if (gm) {
-                            const float gv = load_elem(A.stage_gate_bytes ? gate_stage(st) : gm, A.gate_bf16, gi[v] + e);
-                            add_gated_pair(gv, h, l, tp, tc);
-                        } else {
-                            two_sum(tp, h, tp, qq);
-                            tc = __fadd_rn(tc, __fadd_rn(qq, l));
-                        }
+                    for (int j = 0; j < K; ++j) {
+                        const unsigned char* src = chunk(st, j) + off;
+                        const float f = CB16 ? __uint_as_float((uint32_t)(*reinterpret_cast<const uint16_t*>(src)) << 16)
+                                             : *reinterpret_cast<const float*>(src);
+                        dot2_step(A.w_hi[j], A.w_lo[j], f, p, cc);
                     }
-                    two_sum(tp, tc, hi, lo);
-                };
-                resid_fast<K, U>(A, it, ev, acc, resid, xload, exact, ONE ? A.w_guard[0] : 1.0f);
-            }
+                    two_sum(p, cc, h, l);
+                    // a member without a gate adds like an ungated one (as exact_resid)
+                    const void* gm = GATED ? A.m_gate[first + m] : nullptr;
+                    if (gm) {
+                        const float gv = load_elem(A.stage_gate_bytes ? gate_stage(st) : gm, A.gate_bf16, gi[v] + e);
+                        add_gated_pair(gv, h, l, tp, tc);
+                    } else {
+                        two_sum(tp, h, tp, qq);
+                        tc = __fadd_rn(tc, __fadd_rn(qq, l));
+                    }
+                }
+                two_sum(tp, tc, hi, lo);
+            };
+            resid_fast<K, U>(A, it, ev, acc, resid, xload, exact, ONE ? A.w_guard[0] : 1.0f);
             fence_generic_to_async();
             __syncwarp();
             if (lane == 0)
                 for (int m = 0; m < nb; ++m) mbar_arrive(empty0 + 8u * stage_of(m));
-        } else if (!full_tile) {
-            const long long end = e0 + TE < numel ? e0 + TE : numel;
-            for (long long e = e0 + c; e < end; e += NCT) scalar_element<CB16>(A, K, it, e);
         }
     }
+    return true;
+}
+
+// GROUPED: some item updates a hidden state or has several members (stage
+// holding, hidden-state staging); prediction-only launches compile without
+// that bookkeeping. GATED (with GROUPED): the hidden state receives g_b * P_b,
+// with a per-(batch, channel) gate per member.
+// ONE: the full-step epilogue (copy_out with bf16 hidden states or none): a
+// one-entry history of weight 1, whose member step needs no weighted sum
+// (member_one); PRECISE: fp32 predictions or hidden states; STRIDED: items whose
+// outputs, hidden state or gates are off the 16-byte grid (or whose gate rows
+// hold no whole vectors), every tile by pairs of elements. Compiled apart so
+// that each kernel carries only its own path.
+template <int K, bool CB16, bool GROUPED, bool GATED, bool ONE = false, bool PRECISE = false, bool STRIDED = false>
+__global__ void __launch_bounds__(Shape<CB16, K, GROUPED, GATED, PRECISE>::threads,
+                                  Shape<CB16, K, GROUPED, GATED, PRECISE>::ctas_per_sm)
+    extrapolate_bulk_kernel(const __grid_constant__ ExtrapArgs A) {
+    static_assert(!ONE || (K == 1 && !PRECISE), "the epilogue is a one-entry history");
+    static_assert(!STRIDED || PRECISE, "strided tiles are compensated");
+    extern __shared__ __align__(128) unsigned char smem[];
+    using Sh = Shape<CB16, K, GROUPED, GATED, PRECISE>;
+    constexpr int NCW = Sh::consumer_warps;
+    constexpr long long TE = Sh::tile;
+    const int S = A.stages;
+    const uint32_t full0 = smem_addr(smem);
+    const uint32_t empty0 = full0 + 8u * (uint32_t)S;
+    const uint32_t buf0 = smem_addr(smem + kBarrierBytes);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(full0 + 8u * s, 1);
+            mbar_init(empty0 + 8u * s, NCW);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+
+    // offset of the gate rows in a stage (a grouped launch has hidden states)
+    const uint32_t gates_at =
+        (uint32_t)K * Sh::chunk + (!GROUPED ? 0u : PRECISE ? A.stage_x_bytes : (uint32_t)Sh::tile * 2u);
+    const uint32_t stage_bytes = gates_at + (GATED ? A.stage_gate_bytes : 0u);
+    if (warp == NCW) {
+        if (lane == 0) produce<K, CB16, GROUPED, GATED, PRECISE, STRIDED>(A, full0, empty0, buf0, stage_bytes);
+        return;
+    }
+    const unsigned char* stages = smem + kBarrierBytes;
+    Cursor cur;
+    int tile = blockIdx.x;
+    if constexpr (PRECISE) {
+        int it = 0;
+        for (; tile < A.tiles_total; tile += gridDim.x) {
+            while (tile >= A.tile_begin[it + 1]) ++it;
+            const long long e0 = (long long)(tile - A.tile_begin[it]) * TE;
+            const int n = STRIDED && A.numel[it] - e0 < TE ? (int)(A.numel[it] - e0) : (int)TE;
+            if (!precise_tile<Sh, K, CB16, GROUPED, GATED, STRIDED>(A, it, e0, n, cur, full0, empty0, stages,
+                                                                    stage_bytes, lane))
+                return;
+        }
+        if constexpr (STRIDED) return;
+    } else if (!fast_tiles<K, CB16, GROUPED, GATED, ONE>(A, tile, cur, full0, empty0, stages, stage_bytes, gates_at,
+                                                         lane)) {
+        return;
+    }
+    if (!ragged_tiles<Sh, K, CB16, GROUPED, GATED>(A, tile, cur, full0, empty0, stages, stage_bytes, lane)) return;
+    scalar_items<Sh, K, CB16>(A);
 }
 
 }  // namespace

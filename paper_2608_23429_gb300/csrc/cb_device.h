@@ -33,6 +33,7 @@ struct ExtrapArgs {
     long long slot_off[8];       // byte offset of history entry j (0 = oldest)
     float w_hi[8];               // fp32(w_j)
     float w_lo[8];               // fp32(w_j - w_hi[j])
+    float w_sum;                 // at least sum_j |w_hi[j]|
     float w_guard[8];            // (K+2) u (1.01) 2^9 |w_hi[j]|: the fast path's scaled error bound
     int n_items;
     int tiles_total;
@@ -41,12 +42,16 @@ struct ExtrapArgs {
     int precise;     // 1: compensated (Dot2) arithmetic for every element
     int copy_out;    // full-step epilogue: outputs receive the (K = 1) sources converted, not a prediction
     int stages;                  // bulk variant: shared-memory pipeline depth
-    int stage_chunks;            // bulk variant: 8 KB chunks per stage (K, or K + 1 with hidden states)
-    int stage_x;                 // bulk variant: bf16 hidden states are staged as chunk K
+    unsigned stage_x_bytes;      // bulk variant: bytes of a tile's hidden state staged behind the K chunks (0: not staged)
     unsigned stage_gate_bytes;   // bulk variant: bytes per stage for gate rows (0: gates read from global)
     unsigned long long wait_ns;  // bulk variant: limit of every barrier wait
     int* status;                 // bulk variant: device status word (codes OR-ed in)
     int withhold_first;          // bulk variant, tests only: announce but never issue the first copies
+    // bulk variant: tile_begin and tiles_total count whole tiles only (none of
+    // items with vec_ok = 0); the ragged last tiles are numbered after them
+    int n_ragged;
+    int any_scalar;              // bulk variant: some item has vec_ok = 0
+    short ragged[kMaxItems];     // items with a ragged last tile
     int tile_begin[kMaxItems + 1];
     long long numel[kMaxItems];
     void* resid[kMaxItems];           // hidden state of the item, or null
@@ -82,31 +87,61 @@ constexpr long long push_tile_elems = (long long)kThreads * 2 * kVecElems;
 cudaError_t launch_extrapolate(const ExtrapArgs& a, int K, bool cache_bf16, int grid, cudaStream_t s);
 // gated variant of the direct kernel (extrapolate_gated.cu)
 cudaError_t launch_extrapolate_gated(const ExtrapArgs& a, int K, bool cache_bf16, int grid, cudaStream_t s);
+// with fp32 predictions or hidden states, gated or not (extrapolate_precise.cu)
+cudaError_t launch_extrapolate_precise(const ExtrapArgs& a, int K, bool cache_bf16, bool gated, int grid,
+                                       cudaStream_t s);
 cudaError_t extrapolate_blocks_per_sm(int K, bool cache_bf16, int* blocks);
 
 // Bulk-copy pipeline variant (extrapolate_bulk.cu). Its barrier block holds
 // the full and empty barriers of at most kMaxStages stages.
 constexpr int kMaxStages = 16;
-// CTAs per SM of the bulk kernel (two of 8 consumer warps each, else one):
-// two for K = 1, for bf16 prediction-only launches (not `grouped`) with
+// Shape of the bulk kernel: CTAs per SM, consumer warps of a CTA, elements of
+// a tile.
+//
+// `precise` launches (fp32 predictions or hidden states) are bound by the
+// latency of their arithmetic: as many warps as hold one vector per thread
+// without spilling in the loop, 20 of 96 registers for bf16 sources, 12 of 168
+// for fp32 ones (with the producer a multiple of the four schedulers). GB300,
+// DiT-XL/2 512^2, K = 4, fp32 hidden states, with and without gates: 7 warps
+// 1048 us, 11 871 / 666 us, 15 607 / 509 us, 19 577 / 458 us, 23 (spilling)
+// 746 / 512 us; 11 against 15 warps for fp32 sources, K = 8: 379 / 454 us.
+//
+// Others: two CTAs of 8 consumer warps, else one (16 for bf16 tiles): two
+// for K = 1, for bf16 prediction-only launches (not `grouped`) with
 // K <= 2 and for ungated bf16 grouped launches with K = 2..3, where two
 // vectors per thread still fit the register budget. Ungated bf16 grouped
 // launches with K = 1 (the full-step epilogue from bf16 features) stream
 // faster as one CTA of 16 warps (GB300: FLUX 88.3 -> 94.1 %, DiT-256
 // 81.2 -> 90.1 % of the copy peak, PixArt unchanged); gated ones do not
 // (DiT-256 88.0 -> 63.9 %) and keep two.
-__host__ __device__ constexpr int bulk_ctas_per_sm(int K, bool src_bf16, bool grouped, bool gated) {
-    return ((K == 1 && !(src_bf16 && grouped && !gated)) || (src_bf16 && !grouped && K <= 2) ||
-            (src_bf16 && grouped && !gated && K >= 2 && K <= 3))
-               ? 2
-               : 1;
+struct BulkShape {
+    int ctas_per_sm;
+    int consumer_warps;
+    int tile;
+};
+__host__ __device__ constexpr BulkShape bulk_shape(int K, bool src_bf16, bool grouped, bool gated, bool precise) {
+    if (precise) {
+        const int warps = src_bf16 ? 19 : 11;
+        return BulkShape{1, warps, warps * 32 * kVecElems};
+    }
+    const bool two = (K == 1 && !(src_bf16 && grouped && !gated)) || (src_bf16 && !grouped && K <= 2) ||
+                     (src_bf16 && grouped && !gated && K >= 2 && K <= 3);
+    return BulkShape{two ? 2 : 1, (src_bf16 && !two) ? 16 : 8, (int)tile_elems(src_bf16)};
 }
-size_t bulk_smem_bytes(int chunks_per_stage, size_t extra_per_stage, int stages);
+size_t bulk_smem_bytes(size_t stage_bytes, int stages);
 cudaError_t prepare_extrapolate_bulk(int K, bool cache_bf16, size_t smem);
 // grouped: some item updates a hidden state or has several members (the
 // kernel's hidden-state bookkeeping); it also selects the CTA shape.
 cudaError_t launch_extrapolate_bulk(const ExtrapArgs& a, int K, bool cache_bf16, bool grouped, int grid, size_t smem,
                                     cudaStream_t s);
+// with fp32 predictions or hidden states, gated or not (extrapolate_bulk_precise*.cu)
+cudaError_t prepare_extrapolate_bulk_precise(int K, bool cache_bf16, bool gated, size_t smem);
+cudaError_t launch_extrapolate_bulk_precise(const ExtrapArgs& a, int K, bool cache_bf16, bool grouped, bool gated,
+                                            int grid, size_t smem, cudaStream_t s);
+// for items whose outputs, hidden states or gates are off the 16-byte grid (extrapolate_bulk_strided*.cu)
+cudaError_t prepare_extrapolate_bulk_strided(int K, bool cache_bf16, bool gated, size_t smem);
+cudaError_t launch_extrapolate_bulk_strided(const ExtrapArgs& a, int K, bool cache_bf16, bool grouped, bool gated,
+                                            int grid, size_t smem, cudaStream_t s);
 // gated variant of the bulk kernel (extrapolate_bulk_gated.cu)
 cudaError_t prepare_extrapolate_bulk_gated(int K, bool cache_bf16, size_t smem);
 cudaError_t launch_extrapolate_bulk_gated(const ExtrapArgs& a, int K, bool cache_bf16, int grid, size_t smem,

@@ -14,7 +14,9 @@
 // recomputed from the values already loaded with Dot2 (Ogita, Rump &
 // Oishi, "Accurate Sum and Dot Product", SIAM J. Sci. Comput. 26(6), 2005:
 // TwoProduct by FMA plus TwoSum) with the weights as fp32 pairs hi + lo, and
-// the unevaluated result pair is rounded once. fp32 results always take Dot2.
+// the unevaluated result pair is rounded once. fp32 results always take a
+// compensated sum (sum_vec below): Dot2 for K <= 2, an anchored sum from
+// K = 3 on, both on pairs of elements with packed fp32 operations.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -61,6 +63,19 @@ __device__ __forceinline__ void unpack(const uint4 (&r)[CB16 ? 1 : 2], float (&f
         unpack_f32x8(r[0], r[CB16 ? 0 : 1], f);
 }
 
+// Elements 2q and 2q + 1 of a vector.
+template <bool CB16>
+__device__ __forceinline__ float2 vec_pair(const uint4 (&r)[CB16 ? 1 : 2], int q) {
+    if constexpr (CB16) {
+        const uint32_t w = q == 0 ? r[0].x : q == 1 ? r[0].y : q == 2 ? r[0].z : r[0].w;
+        return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+    } else {
+        const uint4 v = r[(q >> 1) & (CB16 ? 0 : 1)];
+        return (q & 1) ? make_float2(__uint_as_float(v.z), __uint_as_float(v.w))
+                       : make_float2(__uint_as_float(v.x), __uint_as_float(v.y));
+    }
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);  // RNE; .x is the low half
     return *reinterpret_cast<uint32_t*>(&h);
@@ -83,6 +98,19 @@ __device__ __forceinline__ void dot2_step(float w_hi, float w_lo, float f, float
     two_sum(p, h, p, q);
     c = __fadd_rn(c, __fadd_rn(q, r));
     c = __fmaf_rn(w_lo, f, c);
+}
+
+// ---- the same on pairs of elements (packed operations: half the issue slots
+// at the same rate per lane, 115 lane operations per clock and SM measured)
+__device__ __forceinline__ float2 pair_of(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, pair_of(-1.0f), a); }  // a - b, rounded once
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
+    s = add2(a, b);
+    const float2 bb = sub2(s, a);
+    e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
 
 // bf16 of the exact value hi + lo, where hi = fl(hi + lo) (so |lo| <= ulp(hi)/2).
@@ -194,13 +222,13 @@ __device__ __noinline__ void exact_resid(const ExtrapArgs& A, int K, int it, lon
     two_sum(tp, tc, hi, lo);
 }
 
-// One element of item `it` through the compensated path, every member and the
-// hidden state (misaligned items and ragged tails).
+// One element of item `it` through the compensated path, the hidden state and
+// every member (misaligned items and ragged tails).
 template <bool CB16>
 __device__ __noinline__ void scalar_element(const ExtrapArgs& A, int K, int it, long long e) {
     const int first = A.first[it];
     void* resid = A.resid[it];
-    float tp = 0.0f, tc = 0.0f;
+    float tp = resid ? load_elem(resid, A.resid_bf16, e) : 0.0f, tc = 0.0f;
     for (int m = 0; m < A.nb[it]; ++m) {
         float hi, lo, q;
         exact_member<CB16>(A, K, A.m_off[first + m], e, hi, lo);
@@ -217,9 +245,7 @@ __device__ __noinline__ void scalar_element(const ExtrapArgs& A, int K, int it, 
         }
     }
     if (resid) {
-        float q, hi, lo;
-        two_sum(tp, load_elem(resid, A.resid_bf16, e), tp, q);
-        tc = __fadd_rn(tc, q);
+        float hi, lo;
         two_sum(tp, tc, hi, lo);
         store_pair(resid, A.resid_bf16, e, hi, lo);
     }
@@ -247,7 +273,7 @@ __device__ __forceinline__ void store_f32x8(void* p, long long e, const float (&
 
 // Running sums of one item across its members (the fused hidden-state update):
 // fast path x = sum_b s_b, y = sum_b a_b; compensated path x + y is the
-// unevaluated sum (running value and its error).
+// unevaluated sum (running value and its error), begun from the hidden state.
 template <int UV>
 struct Acc {
     float x[UV][8];
@@ -263,30 +289,86 @@ struct Acc {
 template <int K, bool CB16, int UV>
 using RawVecs = uint4[UV][K][CB16 ? 1 : 2];
 
-// Full-step epilogue: the 8 source values of vector (raw) written to out at
-// element e in the output type (see copy_elem).
-template <bool CB16>
-__device__ __forceinline__ void copy_vec(void* out, bool out_bf16, long long e, const uint4 (&r)[CB16 ? 1 : 2]) {
-    if constexpr (CB16) {
-        if (out_bf16) {
-            *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(out) + e) = r[0];
+// Elements 2q, 2q + 1 (the pairs hi + lo, one rounding) into the eight output
+// elements of a vector: fp32 in o[0..7], or bf16 in o[0..3].
+__device__ __forceinline__ void put_pair(uint32_t (&o)[8], bool bf16, int q, float2 hi, float2 lo) {
+    if (bf16) {
+        o[q] = (uint32_t)bf16_of_pair(hi.x, lo.x) | ((uint32_t)bf16_of_pair(hi.y, lo.y) << 16);
+    } else {
+        o[2 * q] = __float_as_uint(hi.x);
+        o[2 * q + 1] = __float_as_uint(hi.y);
+    }
+}
+
+// One pair of output elements e, e + 1 (words w0, w1 as put_pair leaves them);
+// n of the two exist. Adjacent threads hold adjacent pairs.
+__device__ __forceinline__ void store_o2(void* p, bool bf16, long long e, int n, uint32_t w0, uint32_t w1) {
+    if (n <= 0) return;
+    if (bf16) {
+        uint16_t* q = reinterpret_cast<uint16_t*>(p) + e;
+        if (n > 1 && (reinterpret_cast<uintptr_t>(q) & 3) == 0) {
+            *reinterpret_cast<uint32_t*>(q) = w0;
         } else {
-            const uint4 v = r[0];
-            uint4* q = reinterpret_cast<uint4*>(reinterpret_cast<float*>(out) + e);
-            q[0] = make_uint4(v.x << 16, v.x & 0xFFFF0000u, v.y << 16, v.y & 0xFFFF0000u);
-            q[1] = make_uint4(v.z << 16, v.z & 0xFFFF0000u, v.w << 16, v.w & 0xFFFF0000u);
+            q[0] = (uint16_t)w0;
+            if (n > 1) q[1] = (uint16_t)(w0 >> 16);
         }
     } else {
-        const uint4 a = r[0], b = r[CB16 ? 0 : 1];
-        if (out_bf16) {
-            *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(out) + e) = make_uint4(
-                pack_bf16x2(__uint_as_float(a.x), __uint_as_float(a.y)), pack_bf16x2(__uint_as_float(a.z), __uint_as_float(a.w)),
-                pack_bf16x2(__uint_as_float(b.x), __uint_as_float(b.y)), pack_bf16x2(__uint_as_float(b.z), __uint_as_float(b.w)));
+        uint32_t* q = reinterpret_cast<uint32_t*>(p) + e;
+        if (n > 1 && (reinterpret_cast<uintptr_t>(q) & 7) == 0) {
+            *reinterpret_cast<uint2*>(q) = make_uint2(w0, w1);
         } else {
-            uint4* q = reinterpret_cast<uint4*>(reinterpret_cast<float*>(out) + e);
-            q[0] = a;
-            q[1] = b;
+            q[0] = w0;
+            if (n > 1) q[1] = w1;
         }
+    }
+}
+
+__device__ __forceinline__ void store_o8(void* p, bool bf16, long long e, const uint32_t (&o)[8]) {
+    if (bf16) {
+        *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(p) + e) = make_uint4(o[0], o[1], o[2], o[3]);
+    } else {
+        uint4* q = reinterpret_cast<uint4*>(reinterpret_cast<float*>(p) + e);
+        q[0] = make_uint4(o[0], o[1], o[2], o[3]);
+        q[1] = make_uint4(o[4], o[5], o[6], o[7]);
+    }
+}
+
+// Full-step epilogue: the 8 source values of a vector in the output type (see
+// copy_elem): fp32 in o[0..7], or bf16 in o[0..3].
+template <bool CB16>
+__device__ __forceinline__ void copy_o8(bool out_bf16, const uint4 (&r)[CB16 ? 1 : 2], uint32_t (&o)[8]) {
+    const uint4 a = r[0], b = r[CB16 ? 0 : 1];
+    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if constexpr (CB16) {
+            if (out_bf16) {
+                o[i] = w[i];
+            } else {
+                o[2 * i] = w[i] << 16;
+                o[2 * i + 1] = w[i] & 0xFFFF0000u;
+            }
+        } else {
+            if (out_bf16) {
+                o[i] = pack_bf16x2(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1]));
+            } else {
+                o[2 * i] = w[2 * i];
+                o[2 * i + 1] = w[2 * i + 1];
+            }
+        }
+    }
+}
+
+// ... written to out at element e.
+template <bool CB16>
+__device__ __forceinline__ void copy_vec(void* out, bool out_bf16, long long e, const uint4 (&r)[CB16 ? 1 : 2]) {
+    uint32_t o[8];
+    if (out_bf16) {  // two branches with their stores: one store behind a choice of words costs the epilogue 15 %
+        copy_o8<CB16>(true, r, o);
+        store_o8(out, true, e, o);
+    } else {
+        copy_o8<CB16>(false, r, o);
+        store_o8(out, false, e, o);
     }
 }
 
@@ -494,80 +576,189 @@ __device__ __forceinline__ void resid_fast(const ExtrapArgs& A, int it, const lo
     }
 }
 
-// Compensated path for one member (any fp32 prediction or hidden state).
-template <int K, bool CB16, int UV, bool GATED = false, typename Gate = NoGate>
-__device__ __forceinline__ void member_precise(const ExtrapArgs& A, void* out, const long long (&ev)[UV],
-                                               const RawVecs<K, CB16, UV>& raw, bool accumulate,
-                                               Acc<UV>& acc, Gate gate = {}) {
-#pragma unroll
-    for (int u = 0; u < UV; ++u) {
-        float p[8], c[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) p[e] = c[e] = 0.0f;
+// Unevaluated compensated sums s[q] + c[q] = sum_j w_j F_j of the elements
+// 2q, 2q + 1 of one vector.
+//
+// K <= 2: Dot2 (its first TwoSum adds to zero and is left out). K >= 3: an
+// anchored sum. With M = 3 * 2^k, 2^k > W max_j |F_j| and W >= sum_j |w_hi[j]|,
+// every S_j = fl(w_hi[j] F_j + S_{j-1}), S_{-1} = M, stays in the binade of M,
+// so d_j = S_j - S_{j-1} is exact, and what the rounding left out,
+// w_hi[j] F_j - d_j (at most half a unit of M), is one FMA; c collects it with
+// the weight's low half. S_{K-1} - M is exact (the error-free extraction by a
+// large constant of Rump, Ogita & Oishi, "Accurate floating-point summation",
+// SIAM J. Sci. Comput. 31(1), 2008, with the product folded into the FMA).
+// Five operations per term against Dot2's eleven: with fp32 results the
+// kernels are bound by the FMA pipe. s + c is within 2^-40 sum_j |w_j F_j| of
+// the exact value (Dot2: 2^-45; 2^6 million sums, K = 3..8, bf16 and fp32
+// features), and the fp32 results' 2-norm error equals Dot2's to seven digits.
+// Where M overflows (W max |F| >= 2^126) or a feature is not finite, s is not
+// finite: the callers then take scalar_element, which has no anchor.
+//
+// Two pairs advance together, term by term (four at once take registers from
+// the other warps; one at a time is as fast with five warps per scheduler).
+template <int K, bool CB16>
+__device__ __forceinline__ void sum_vec(const ExtrapArgs& A, const uint4 (&raw)[K][CB16 ? 1 : 2], float2 (&s)[4],
+                                        float2 (&c)[4]) {
+    if constexpr (K <= 2) {
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            float f[8];
-            unpack<CB16>(raw[u][j], f);
+            const float2 w = pair_of(A.w_hi[j]), wl = pair_of(A.w_lo[j]);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) dot2_step(A.w_hi[j], A.w_lo[j], f[e], p[e], c[e]);
-        }
-        float hi[8], lo[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) two_sum(p[e], c[e], hi[e], lo[e]);
-        if (out) {
-            if (A.out_bf16) {
-                uint32_t pk[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    pk[i] = (uint32_t)bf16_of_pair(hi[2 * i], lo[2 * i]) |
-                            ((uint32_t)bf16_of_pair(hi[2 * i + 1], lo[2 * i + 1]) << 16);
-                store_bf16x8(out, ev[u], pk);
-            } else {
-                store_f32x8(out, ev[u], hi);
+            for (int q = 0; q < 4; ++q) {
+                const float2 f = vec_pair<CB16>(raw[j], q);
+                if (j == 0) {
+                    s[q] = mul2(w, f);
+                    c[q] = fma2(w, f, mul2(pair_of(-A.w_hi[j]), f));  // exact: w_hi*f - s
+                } else {
+                    const float2 h = mul2(w, f);
+                    float2 e;
+                    two_sum2(s[q], h, s[q], e);
+                    c[q] = add2(c[q], add2(e, fma2(w, f, mul2(pair_of(-A.w_hi[j]), f))));
+                }
+                c[q] = fma2(wl, f, c[q]);
             }
         }
-        if (accumulate) {
-            float g[8];
-            if constexpr (GATED) gate(u, g);
+    } else {
+        float2 anchor[4];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                if constexpr (GATED) {
-                    add_gated_pair(g[e], hi[e], lo[e], acc.x[u][e], acc.y[u][e]);
+        for (int q0 = 0; q0 < 4; q0 += 2) {
+#pragma unroll
+            for (int q = q0; q < q0 + 2; ++q) {
+                float2 m;
+                if constexpr (CB16) {  // the signs of m are of no account: only its exponents are used
+                    uint32_t x = q == 0 ? raw[0][0].x : q == 1 ? raw[0][0].y : q == 2 ? raw[0][0].z : raw[0][0].w;
+#pragma unroll
+                    for (int j = 1; j < K; ++j) {
+                        const uint4 v = raw[j][0];
+                        asm("max.xorsign.abs.bf16x2 %0, %0, %1;"
+                            : "+r"(x)
+                            : "r"(q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w));
+                    }
+                    m = make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u));
                 } else {
-                    float q;
-                    two_sum(acc.x[u][e], hi[e], acc.x[u][e], q);
-                    acc.y[u][e] = __fadd_rn(acc.y[u][e], __fadd_rn(q, lo[e]));
+                    m = vec_pair<CB16>(raw[0], q);
+#pragma unroll
+                    for (int j = 1; j < K; ++j) {
+                        const float2 f = vec_pair<CB16>(raw[j], q);
+                        m = make_float2(fmaxf(fabsf(m.x), fabsf(f.x)), fmaxf(fabsf(m.y), fabsf(f.y)));
+                    }
+                }
+                const float2 v = mul2(pair_of(A.w_sum), m);
+                anchor[q] = mul2(make_float2(__uint_as_float(__float_as_uint(v.x) & 0x7F800000u),
+                                             __uint_as_float(__float_as_uint(v.y) & 0x7F800000u)),
+                                 pair_of(6.0f));
+                s[q] = anchor[q];
+            }
+#pragma unroll
+            for (int j = 0; j < K; ++j) {
+                const float2 w = pair_of(A.w_hi[j]), wl = pair_of(A.w_lo[j]);
+#pragma unroll
+                for (int q = q0; q < q0 + 2; ++q) {
+                    const float2 f = vec_pair<CB16>(raw[j], q);
+                    const float2 t = fma2(w, f, s[q]);
+                    const float2 r = fma2(w, f, sub2(s[q], t));
+                    c[q] = fma2(wl, f, j == 0 ? r : add2(c[q], r));
+                    s[q] = t;
                 }
             }
+#pragma unroll
+            for (int q = q0; q < q0 + 2; ++q) s[q] = sub2(s[q], anchor[q]);
         }
     }
 }
 
-template <int UV, typename XLoad>
-__device__ __forceinline__ void resid_precise(const ExtrapArgs& A, const long long (&ev)[UV], Acc<UV>& acc,
-                                              void* resid, XLoad xload) {
+// Finiteness of a thread's compensated results: `zero` stays +-0 exactly as
+// long as every value given to it is finite.
+struct Finite {
+    float2 zero = {0.0f, 0.0f};
+    __device__ __forceinline__ void see(float2 v) { zero = fma2(v, pair_of(0.0f), zero); }
+    __device__ __forceinline__ bool all() const { return zero.x == 0.0f && zero.y == 0.0f; }
+};
+
+// Compensated path for one member (any launch with fp32 predictions or hidden
+// states): the prediction's output elements to put(u, o) when wanted (o as
+// put_pair leaves it, for vector u), and accumulation into acc.
+template <int K, bool CB16, int UV, bool GATED, typename Gate, typename Put>
+__device__ __forceinline__ void member_precise(const ExtrapArgs& A, bool want, const RawVecs<K, CB16, UV>& raw,
+                                               bool accumulate, Acc<UV>& acc, Finite& fin, Gate gate, Put put) {
 #pragma unroll
     for (int u = 0; u < UV; ++u) {
-        float x[8], hi[8], lo[8];
-        xload(u, x);
+        uint32_t o[8];
+        float2 sv[4], cv[4];
+        sum_vec<K, CB16>(A, raw[u], sv, cv);
+        float g[8];
+        if constexpr (GATED)
+            if (accumulate) gate(u, g);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            float q;
-            two_sum(acc.x[u][e], x[e], acc.x[u][e], q);
-            acc.y[u][e] = __fadd_rn(acc.y[u][e], q);
-            two_sum(acc.x[u][e], acc.y[u][e], hi[e], lo[e]);
+        for (int q = 0; q < 4; ++q) {
+            const float2 s = sv[q], c = cv[q];
+            if (want) {
+                if (A.out_bf16) {
+                    float2 hi, lo;
+                    two_sum2(s, c, hi, lo);
+                    put_pair(o, true, q, hi, lo);
+                    if (K > 2) fin.see(hi);
+                } else {
+                    const float2 hi = add2(s, c);
+                    put_pair(o, false, q, hi, hi);
+                    if (K > 2) fin.see(hi);
+                }
+            }
+            if (accumulate) {
+                float2 x = make_float2(acc.x[u][2 * q], acc.x[u][2 * q + 1]);
+                float2 y = make_float2(acc.y[u][2 * q], acc.y[u][2 * q + 1]), e;
+                if constexpr (GATED) {
+                    const float2 gq = make_float2(g[2 * q], g[2 * q + 1]);
+                    const float2 gs = mul2(gq, s);
+                    const float2 gr = fma2(gq, s, make_float2(-gs.x, -gs.y));  // exact: g*s - gs
+                    two_sum2(x, gs, x, e);
+                    y = fma2(gq, c, add2(y, add2(e, gr)));
+                } else {
+                    two_sum2(x, s, x, e);
+                    y = add2(y, add2(e, c));
+                }
+                acc.x[u][2 * q] = x.x;
+                acc.x[u][2 * q + 1] = x.y;
+                acc.y[u][2 * q] = y.x;
+                acc.y[u][2 * q + 1] = y.y;
+            }
         }
-        if (A.resid_bf16) {
-            uint32_t pk[4];
+        if (want) put(u, o);
+    }
+}
+
+// The compensated sums start from the hidden state (xload(u, x), as resid_fast).
+template <int UV, typename XLoad>
+__device__ __forceinline__ void resid_begin(Acc<UV>& acc, XLoad xload) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                pk[i] = (uint32_t)bf16_of_pair(hi[2 * i], lo[2 * i]) |
-                        ((uint32_t)bf16_of_pair(hi[2 * i + 1], lo[2 * i + 1]) << 16);
-            store_bf16x8(resid, ev[u], pk);
-        } else {
-            store_f32x8(resid, ev[u], hi);
+    for (int u = 0; u < UV; ++u) {
+        xload(u, acc.x[u]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc.y[u][e] = 0.0f;
+    }
+}
+
+// Rounds the compensated hidden state to put(u, o), unless a result was not
+// finite (then nothing is stored and the caller recomputes the elements).
+template <int K, int UV, typename Put>
+__device__ __forceinline__ bool resid_precise(const ExtrapArgs& A, const Acc<UV>& acc, Finite& fin, Put put) {
+    uint32_t o[UV][8];
+#pragma unroll
+    for (int u = 0; u < UV; ++u) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2 x = make_float2(acc.x[u][2 * q], acc.x[u][2 * q + 1]);
+            const float2 y = make_float2(acc.y[u][2 * q], acc.y[u][2 * q + 1]);
+            float2 hi, lo;
+            two_sum2(x, y, hi, lo);
+            put_pair(o[u], A.resid_bf16, q, hi, lo);
+            if (K > 2) fin.see(hi);
         }
     }
+    if (K > 2 && !fin.all()) return false;
+#pragma unroll
+    for (int u = 0; u < UV; ++u) put(u, o[u]);
+    return true;
 }
 
 // n / d for n, d < 2^32 from M = ceil(2^64 / d) (M = 0 encodes d = 1):
@@ -592,17 +783,39 @@ __device__ __forceinline__ void gate_offsets(const ExtrapArgs& A, int it, long l
         for (int u = 0; u < UV; ++u) gi[u] = 0;
         return;
     }
+    // what the tile's first element fixes is the same for every thread; a
+    // thread's own channel is (h0 + d) mod H for its offset d in the tile. With
+    // m = ceil(2^32 / H), x < 2^32 / H has x / H = x m / 2^32 exactly (as in
+    // div_magic), and wider rows than that hold a tile, so that x < 2 H.
     const unsigned q0 = div_magic(ue0, A.i_row_magic[it]), r0 = ue0 - q0 * row;
+    const unsigned h0 = r0 - div_magic(r0, A.i_hidden_magic[it]) * H;
+    const unsigned m32 = (unsigned)((A.i_hidden_magic[it] + 0xFFFFFFFFull) >> 32);
 #pragma unroll
     for (int u = 0; u < UV; ++u) {
-        unsigned r = r0 + (unsigned)(ev[u] - e0), b = relative ? 0u : q0;
+        const unsigned d = (unsigned)(ev[u] - e0), x = h0 + d;
+        unsigned h;
+        if (H > 16384u)
+            h = x >= H ? x - H : x;
+        else
+            h = m32 ? x - __umulhi(x, m32) * H : 0u;
+        unsigned r = r0 + d, b = relative ? 0u : q0;
         while (r >= row) {  // a tile spans few rows
             r -= row;
             ++b;
         }
-        const unsigned h = r - div_magic(r, A.i_hidden_magic[it]) * H;
         gi[u] = b * H + h;
     }
+}
+
+// Gate offsets of the elements e and e + 1 (32-bit, as above; e + 1 may lie in
+// the next channel row, token or batch). The item has a shape.
+__device__ __forceinline__ void gate_offset_pair(const ExtrapArgs& A, int it, long long e, unsigned& g0, unsigned& g1) {
+    const unsigned row = A.i_row[it], H = A.i_hidden[it], ue = (unsigned)e;
+    const unsigned b = div_magic(ue, A.i_row_magic[it]), r = ue - b * row;
+    const unsigned h = r - div_magic(r, A.i_hidden_magic[it]) * H;
+    g0 = b * H + h;
+    g1 = g0 + 1;
+    if (h + 1 == H && r + 1 < row) g1 -= H;  // the next token of the same batch
 }
 
 // The 8 gate values of member mi for each of UV vectors (1 without a gate).

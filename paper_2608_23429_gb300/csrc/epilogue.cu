@@ -17,8 +17,9 @@
 // compensated path throughout, aside).
 //
 // Each thread has (members + 1) loads in flight, so the kernel streams well
-// only when groups are large: the host runs it for ungated bf16 features when
-// every tensor belongs to a residual group of three or more branches (GB300,
+// only when groups are large: the host runs it for ungated bf16 features and
+// bf16 hidden states when every tensor belongs to a residual group of three or
+// more branches (GB300,
 // PixArt-Sigma 1024^2, groups of 3: 96.1 % of the copy peak against 91.4 % for
 // the bulk pipeline; FLUX.1-dev, groups of 1 and 2: 82.4 % against 93.9 %).
 #include "direct_kernel.cuh"
@@ -42,9 +43,8 @@ __device__ __forceinline__ void epilogue_vector(const ExtrapArgs& A, int it, con
 #pragma unroll
     for (int m = 0; m < kEpilogueMaxMembers; ++m)
         if (m < nb) load_member<1, CB16, 1>(A, A.m_off[first + m], ev, raw[m]);
-    const bool x16 = resid != nullptr && A.resid_bf16;
     uint4 xr = make_uint4(0u, 0u, 0u, 0u);
-    if (x16) xr = ld_v4(reinterpret_cast<const unsigned char*>(resid) + ev[0] * 2);
+    if (resid) xr = ld_v4(reinterpret_cast<const unsigned char*>(resid) + ev[0] * 2);
     unsigned gi[1] = {0u};
     if constexpr (GATED) {  // items without shapes carry no gate
         if (resid && A.i_hidden[it] != 0) gate_offsets<1>(A, it, ev[0], ev, gi);
@@ -64,28 +64,16 @@ __device__ __forceinline__ void epilogue_vector(const ExtrapArgs& A, int it, con
 #pragma unroll
                 for (int e = 0; e < 8; ++e) gv[e] = 1.0f;
         };
-        if (A.precise)
-            member_precise<1, CB16, 1, GATED>(A, nullptr, ev, raw[m], true, acc, gate);
-        else if constexpr (CB16)  // bf16 features: exact, no weighted sum
+        if constexpr (CB16)  // bf16 features: exact, no weighted sum
             member_one<1, CB16, 1, GATED>(raw[m], acc, gate);
         else
             member_fast<1, CB16, 1, false, GATED>(A, A.m_off[first + m], nullptr, ev, raw[m], true, acc, gate);
     }
     if (!resid) return;
-    auto xload = [&](int, float (&x)[8]) {
-        if (x16)
-            unpack_bf16x8(xr, x);
-        else
-            load_x8(resid, false, ev[0], x);
-    };
-    if (A.precise) {
-        resid_precise<1>(A, ev, acc, resid, xload);
-    } else {
-        resid_fast<1, 1>(
-            A, it, ev, acc, resid, xload,
-            [&](int, int e, float xe, float& hi, float& lo) { exact_resid<CB16>(A, 1, it, ev[0] + e, xe, hi, lo); },
-            CB16 ? A.w_guard[0] : 1.0f);
-    }
+    resid_fast<1, 1>(
+        A, it, ev, acc, resid, [&](int, float (&x)[8]) { unpack_bf16x8(xr, x); },
+        [&](int, int e, float xe, float& hi, float& lo) { exact_resid<CB16>(A, 1, it, ev[0] + e, xe, hi, lo); },
+        CB16 ? A.w_guard[0] : 1.0f);
 }
 
 template <bool CB16, bool GATED>

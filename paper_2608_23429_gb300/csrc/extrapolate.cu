@@ -6,13 +6,13 @@ namespace {
 
 template <int K, bool CB16>
 cudaError_t launch_k(const ExtrapArgs& a, int grid, cudaStream_t s) {
-    extrapolate_kernel<K, CB16, false><<<grid, kThreads, 0, s>>>(a);
+    extrapolate_kernel<K, CB16, false, false><<<grid, kThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 template <int K, bool CB16>
 cudaError_t occ_k(int* blocks) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, extrapolate_kernel<K, CB16, false>, kThreads, 0);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, extrapolate_kernel<K, CB16, false, false>, kThreads, 0);
 }
 
 template <bool CB16>

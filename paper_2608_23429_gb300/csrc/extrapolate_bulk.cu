@@ -9,20 +9,19 @@ namespace {
 template <int K, bool CB16, bool ONE>
 cudaError_t launch_kk(const ExtrapArgs& a, bool grouped, int grid, size_t smem, cudaStream_t s) {
     if (grouped)
-        extrapolate_bulk_kernel<K, CB16, true, false, ONE><<<grid, Shape<CB16, K, true, false>::threads, smem, s>>>(a);
+        extrapolate_bulk_kernel<K, CB16, true, false, ONE><<<grid, Shape<CB16, K, true, false, false>::threads, smem, s>>>(a);
     else
-        extrapolate_bulk_kernel<K, CB16, false, false, ONE><<<grid, Shape<CB16, K, false, false>::threads, smem, s>>>(a);
+        extrapolate_bulk_kernel<K, CB16, false, false, ONE><<<grid, Shape<CB16, K, false, false, false>::threads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
-// The full-step epilogue from bf16 features (a copy_out launch without
-// compensated hidden states) runs the ONE instantiations. From fp32 features
+// The full-step epilogue from bf16 features (a copy_out launch) runs the ONE instantiations. From fp32 features
 // the general path measured faster on GB300 (FLUX 95.6 % against 89.0 % of the
 // copy peak), so those launches keep it.
 template <int K, bool CB16>
 cudaError_t launch_k(const ExtrapArgs& a, bool grouped, int grid, size_t smem, cudaStream_t s) {
     if constexpr (K == 1 && CB16)
-        if (a.copy_out && !a.precise) return launch_kk<K, CB16, true>(a, grouped, grid, smem, s);
+        if (a.copy_out) return launch_kk<K, CB16, true>(a, grouped, grid, smem, s);
     return launch_kk<K, CB16, false>(a, grouped, grid, smem, s);
 }
 
@@ -58,9 +57,7 @@ cudaError_t prepare_k(size_t smem) {
 
 }  // namespace
 
-size_t bulk_smem_bytes(int chunks_per_stage, size_t extra_per_stage, int stages) {
-    return kBarrierBytes + (size_t)stages * ((size_t)chunks_per_stage * kChunkBytes + extra_per_stage);
-}
+size_t bulk_smem_bytes(size_t stage_bytes, int stages) { return kBarrierBytes + (size_t)stages * stage_bytes; }
 
 cudaError_t prepare_extrapolate_bulk(int K, bool cache_bf16, size_t smem) {
 #define P_BF(k) prepare_k<k, true>(smem)

@@ -7,7 +7,7 @@ namespace {
 
 template <int K, bool CB16>
 cudaError_t launch_gk(const ExtrapArgs& a, int grid, cudaStream_t s) {
-    extrapolate_kernel<K, CB16, true><<<grid, kThreads, 0, s>>>(a);
+    extrapolate_kernel<K, CB16, true, false><<<grid, kThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

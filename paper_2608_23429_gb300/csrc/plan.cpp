@@ -69,6 +69,8 @@ struct DeviceInfo {
     int occ_epilogue = 0;                  // epilogue kernel (bf16 features, no gates)
     int bulk_stages[2][CB_MAX_K + 1] = {};  // 1 once the kernel's shared-memory limit is raised
     int bulk_gated[2][CB_MAX_K + 1] = {};   // the same for the gated kernel
+    int bulk_precise[2][2][CB_MAX_K + 1] = {};  // [gated]: the same for fp32 predictions or hidden states
+    int bulk_strided[2][2][CB_MAX_K + 1] = {};  // [gated]: the same for items off the 16-byte grid
 };
 
 }  // namespace
@@ -103,6 +105,7 @@ struct cb_plan {
     DeviceInfo dev;
     // value-initialised: no field of a launch's arguments is ever left unset
     std::unique_ptr<cbk::ExtrapArgs> eargs{new cbk::ExtrapArgs()};
+    std::unique_ptr<cbk::ExtrapArgs> eargs2;  // part of a call's items (made when first needed)
     std::unique_ptr<cbk::PushArgs> pargs{new cbk::PushArgs()};
 
     double tau(double t) const { return 2.0 * (t - t_min) / (t_max - t_min) - 1.0; }
@@ -147,30 +150,35 @@ int extrap_grid(cb_plan* p, int K, bool cb16, int tiles, int* grid) {
 // Largest gate staging per pipeline stage (two rows of 4096 fp32 channels).
 constexpr size_t kMaxStagedGateBytes = 32768;
 
-// Pipeline of the bulk kernel: as many stages of `chunks` 8 KB chunks (plus
-// `extra` bytes) as fit in one CTA's shared memory, at most kMaxStages, and
-// the CTAs per SM. A shape made for two CTAs per SM runs one, with all of the
-// SM's shared memory, when half of it cannot hold `min_stages`. The kernel's
-// dynamic shared-memory limit is raised to the device maximum once per
-// instantiation.
-int bulk_config(cb_plan* p, int K, bool cb16, bool grouped, int chunks, size_t extra, bool gated, int min_stages,
-                int* stages, size_t* smem, int* ctas_per_sm) {
-    int& prepared = gated ? p->dev.bulk_gated[cb16 ? 1 : 0][K] : p->dev.bulk_stages[cb16 ? 1 : 0][K];
+// Pipeline of the bulk kernel: as many stages of `stage_bytes` as fit in one
+// CTA's shared memory, at most kMaxStages, and the CTAs per SM. A shape made
+// for two CTAs per SM runs one, with all of the SM's shared memory, when half
+// of it cannot hold `min_stages`. The kernel's dynamic shared-memory limit is
+// raised to the device maximum once per instantiation.
+int bulk_config(cb_plan* p, int K, bool cb16, bool gated, bool precise, bool strided, int shape_ctas,
+                size_t stage_bytes, int min_stages, int* stages, size_t* smem, int* ctas_per_sm) {
+    int& prepared = strided ? p->dev.bulk_strided[gated ? 1 : 0][cb16 ? 1 : 0][K]
+                    : precise ? p->dev.bulk_precise[gated ? 1 : 0][cb16 ? 1 : 0][K]
+                    : gated ? p->dev.bulk_gated[cb16 ? 1 : 0][K]
+                            : p->dev.bulk_stages[cb16 ? 1 : 0][K];
     if (prepared == 0) {
-        cudaError_t e = gated ? cbk::prepare_extrapolate_bulk_gated(K, cb16, (size_t)p->dev.smem_optin)
-                              : cbk::prepare_extrapolate_bulk(K, cb16, (size_t)p->dev.smem_optin);
+        const size_t most = (size_t)p->dev.smem_optin;
+        cudaError_t e = strided   ? cbk::prepare_extrapolate_bulk_strided(K, cb16, gated, most)
+                        : precise ? cbk::prepare_extrapolate_bulk_precise(K, cb16, gated, most)
+                        : gated ? cbk::prepare_extrapolate_bulk_gated(K, cb16, most)
+                                : cbk::prepare_extrapolate_bulk(K, cb16, most);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
         prepared = 1;
     }
     // with several CTAs per SM each gets its share of the SM's shared memory
     // (less the 1 KB the hardware reserves per CTA)
-    for (int per_sm = cbk::bulk_ctas_per_sm(K, cb16, grouped, gated); per_sm >= 1; --per_sm) {
+    for (int per_sm = shape_ctas; per_sm >= 1; --per_sm) {
         size_t cap = (size_t)p->dev.smem_optin;
         if (per_sm > 1) cap = std::min(cap, (size_t)p->dev.smem_per_sm / per_sm - 1024);
         int s = cbk::kMaxStages;
-        while (s > 1 && cbk::bulk_smem_bytes(chunks, extra, s) > cap) --s;
-        *stages = cbk::bulk_smem_bytes(chunks, extra, s) <= cap ? s : 0;
-        *smem = cbk::bulk_smem_bytes(chunks, extra, s);
+        while (s > 1 && cbk::bulk_smem_bytes(stage_bytes, s) > cap) --s;
+        *stages = cbk::bulk_smem_bytes(stage_bytes, s) <= cap ? s : 0;
+        *smem = cbk::bulk_smem_bytes(stage_bytes, s);
         *ctas_per_sm = per_sm;
         if (*stages >= min_stages) break;
     }
@@ -300,6 +308,225 @@ int clear_word(int* word, void* stream) {
     return e == cudaSuccess ? CB_OK : cuda_fail(e, "cudaMemsetAsync");
 }
 
+// What the launches of one call share.
+struct Launch {
+    cb_plan* p;
+    int K;
+    bool cb16;         // source type: bf16 (else fp32)
+    bool full_step;    // the sources are a full step's new features
+    size_t res;        // bytes of a hidden-state element
+    cb_dtype gate_dtype;
+    void* stream;
+    CallerHistory* ch;
+    bool cleared = false;
+};
+
+int clear_status(Launch& L) {
+    if (!L.ch) return clear_status_once(L.p, L.stream);
+    if (L.cleared) return CB_OK;
+    const int r = clear_word(L.ch->status, L.stream);
+    L.ch->launched = L.cleared = r == CB_OK;
+    return r;
+}
+
+// Cut the items into tiles of te elements, numbered across items. `split` (the
+// bulk kernel's numbering): whole tiles first, then the ragged last ones;
+// items off the 16-byte grid have none.
+int cut_tiles(cbk::ExtrapArgs& A, long long te, bool split) {
+    long long tiles = 0;
+    A.n_ragged = A.any_scalar = 0;
+    for (int i = 0; i < A.n_items; ++i) {
+        A.tile_begin[i] = (int)tiles;
+        if (split && !A.vec_ok[i]) {
+            A.any_scalar = 1;
+            continue;
+        }
+        if (split && A.numel[i] % te != 0) A.ragged[A.n_ragged++] = (short)i;
+        tiles += split ? A.numel[i] / te : (A.numel[i] + te - 1) / te;
+        if (tiles + A.n_ragged > 0x7FFFFFFFLL) return CB_ERR_LIMIT;
+    }
+    A.tile_begin[A.n_items] = A.tiles_total = (int)tiles;
+    return CB_OK;
+}
+
+bool any_gate(const cbk::ExtrapArgs& A) {
+    for (int i = 0; i < A.n_items; ++i)
+        for (int m = 0; m < A.nb[i]; ++m)
+            if (A.m_gate[A.first[i] + m]) return true;
+    return false;
+}
+
+// The items of A whose flag is `want`, with their members, as B.
+void take_items(const cbk::ExtrapArgs& A, const bool* flag, bool want, cbk::ExtrapArgs& B) {
+    B = A;
+    B.n_items = 0;
+    int members = 0;
+    for (int i = 0; i < A.n_items; ++i) {
+        if (flag[i] != want) continue;
+        const int k = B.n_items++;
+        B.numel[k] = A.numel[i];
+        B.resid[k] = A.resid[i];
+        B.nb[k] = A.nb[i];
+        B.vec_ok[k] = A.vec_ok[i];
+        B.first[k] = (short)members;
+        B.i_hidden[k] = A.i_hidden[i];
+        B.i_row[k] = A.i_row[i];
+        B.i_hidden_magic[k] = A.i_hidden_magic[i];
+        B.i_row_magic[k] = A.i_row_magic[i];
+        for (int m = 0; m < A.nb[i]; ++m, ++members) {
+            B.m_off[members] = A.m_off[A.first[i] + m];
+            B.m_out[members] = A.m_out[A.first[i] + m];
+            B.m_gate[members] = A.m_gate[A.first[i] + m];
+        }
+    }
+}
+
+int launch_direct(Launch& L, cbk::ExtrapArgs& A) {
+    int grid = 0;
+    int r = cut_tiles(A, cbk::tile_elems(L.cb16), false);
+    if (r == CB_OK) r = extrap_grid(L.p, L.K, L.cb16, A.tiles_total, &grid);
+    if (r == CB_OK) r = clear_status(L);
+    if (r != CB_OK) return r;
+    const cudaStream_t s = (cudaStream_t)L.stream;
+    const bool gated = any_gate(A);
+    cudaError_t e = A.precise ? cbk::launch_extrapolate_precise(A, L.K, L.cb16, gated, grid, s)
+                    : gated   ? cbk::launch_extrapolate_gated(A, L.K, L.cb16, grid, s)
+                              : cbk::launch_extrapolate(A, L.K, L.cb16, grid, s);
+    return e == cudaSuccess ? CB_OK : cuda_fail(e, "extrapolate launch");
+}
+
+int launch_epilogue(Launch& L, cbk::ExtrapArgs& A) {
+    int& occ = L.p->dev.occ_epilogue;
+    if (occ == 0) {
+        cudaError_t e = cbk::epilogue_blocks_per_sm(&occ);
+        if (e != cudaSuccess || occ <= 0) {
+            occ = 0;
+            return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "occupancy");
+        }
+    }
+    int r = cut_tiles(A, cbk::epilogue_tile_elems, false);
+    if (r == CB_OK) r = clear_status(L);
+    if (r != CB_OK) return r;
+    const int grid = (int)std::min<long long>(A.tiles_total, (long long)L.p->dev.sms * occ);
+    cudaError_t e = cbk::launch_epilogue(A, grid, (cudaStream_t)L.stream);
+    return e == cudaSuccess ? CB_OK : cuda_fail(e, "epilogue launch");
+}
+
+// The bulk-copy pipeline. `strided`: every item is off the 16-byte grid on its
+// way out (see the kernel's STRIDED).
+int launch_bulk(Launch& L, cbk::ExtrapArgs& A, bool strided) {
+    cb_plan* p = L.p;
+    const int K = L.K, items = A.n_items;
+    const bool cb16 = L.cb16, gated = any_gate(A), precise = A.precise != 0 || strided;
+    // the grouped kernel (hidden-state bookkeeping) for gates, hidden states or multi-member items
+    int max_nb = 1;
+    bool grouped = gated, any_resid = false;
+    for (int i = 0; i < items; ++i) {
+        max_nb = std::max(max_nb, (int)A.nb[i]);
+        any_resid = any_resid || A.resid[i] != nullptr;
+        grouped = grouped || A.resid[i] != nullptr || A.nb[i] > 1;
+    }
+    const cbk::BulkShape shape = cbk::bulk_shape(K, cb16, grouped, gated, precise);
+    int rc = cut_tiles(A, shape.tile, !strided);
+    if (rc != CB_OK) return rc;
+    // Hidden states travel through shared memory with the first member of their
+    // group (not those off the 16-byte grid). Launches that recompute guarded
+    // elements hold a whole group and need one stage ahead of it; compensated
+    // ones hold nothing.
+    A.stage_x_bytes = any_resid && !strided ? (unsigned)(shape.tile * L.res) : 0u;
+    A.stage_gate_bytes = 0;
+    const bool hold = grouped && !precise;
+    const int min_stages = hold ? max_nb + 1 : 2;
+    // gate rows travel with their member when every gated tile touches at
+    // most two batches (a batch holds a tile or more) and two rows are small
+    if (gated && !precise) {
+        const size_t gs = esize(L.gate_dtype);
+        size_t need = 0;
+        bool fits = true;
+        for (int i = 0; i < items; ++i) {
+            bool gated_item = false;
+            for (int m = 0; m < A.nb[i]; ++m) gated_item = gated_item || A.m_gate[A.first[i] + m];
+            if (!gated_item || !A.vec_ok[i]) continue;
+            fits = fits && (long long)A.i_row[i] >= shape.tile;
+            need = std::max(need, 2 * (size_t)A.i_hidden[i] * gs);
+        }
+        if (fits && need <= kMaxStagedGateBytes) A.stage_gate_bytes = (unsigned)((need + 127) / 128 * 128);
+    }
+    size_t smem = 0;
+    int per_sm = 1;
+    const size_t stage_bytes =
+        (size_t)K * shape.tile * esize(cb16 ? CB_BF16 : CB_FP32) + A.stage_x_bytes + A.stage_gate_bytes;
+    rc = bulk_config(p, K, cb16, gated, precise, strided, shape.ctas_per_sm, stage_bytes, min_stages, &A.stages, &smem,
+                     &per_sm);
+    if (rc != CB_OK) return rc;
+    if (A.stages < min_stages) {  // too deep for shared memory
+        // A group too large to hold: the compensated kernels hold none (GB300,
+        // 10 groups of 4 x [8, 256, 1152], K = 8: 290 us against 318 us for the
+        // direct-load kernel, 329 against 458 us with gates; fp32 sources, 5
+        // groups of 4 x [4, 256, 1152], K = 6..8: 102, 112, 125 against 109,
+        // 129, 139 us). bf16 sources with K <= 6 are faster there (33 groups of
+        // 4 x [4, 409, 1016], K = 6, gates: 515 against 604 us).
+        if (!hold || (cb16 && K <= 6)) return launch_direct(L, A);
+        A.precise = 1;
+        return launch_bulk(L, A, false);
+    }
+    const int stages_all = A.stages;
+    const size_t smem_all = smem;
+    // Bytes in flight. HBM serves a mix of reads and writes best when no more is
+    // asked of it than covers its latency; beyond that reads and writes turn
+    // the bus around more often. GB300, DiT-XL/2 256^2 shapes, every SM, KB in
+    // flight per SM (all that fits -> here): predictions with K = 1 100.0 ->
+    // 83.8 us (48), K = 2 136 -> 120 (64), K = 3 169 -> 151 (120), K = 4 206 ->
+    // 188 (128); full-step epilogue from fp32 features 176 -> 159 (100). The
+    // more is read per byte written, the flatter the optimum and the higher.
+    // Launches that hold a group's stages keep two groups' worth; those with
+    // K >= 2 are bound by their consumers and any depth serves them.
+    if (!hold || K == 1) {
+        double rd = 0, wr = 0, units = 0;
+        for (int i = 0; i < items; ++i) {
+            const double e = (double)A.numel[i], x = A.resid[i] ? (double)L.res : 0.0;
+            rd += e * (A.nb[i] * K * (cb16 ? 2.0 : 4.0) + x);
+            units += e * A.nb[i];
+            wr += e * x;
+            for (int m = 0; m < A.nb[i]; ++m)
+                if (A.m_out[A.first[i] + m]) wr += e * (A.out_bf16 ? 2.0 : 4.0);
+        }
+        const double ratio = rd / wr, kb = hold ? 76 : ratio < 1.25 ? 48 : ratio < 2.5 ? 76 : 120;
+        const double unit = rd / units * shape.tile;
+        const int most = (int)(kb * 1024.0 / unit / per_sm + 0.5);
+        const int least = std::max(hold ? 2 * max_nb : 2, per_sm == 1 ? 3 : 2);
+        A.stages = std::min(A.stages, std::max(most, least));
+        smem = cbk::bulk_smem_bytes(stage_bytes, A.stages);
+    }
+    // Persistent grid: every SM, except that bf16 prediction-only launches with
+    // K = 5 and 6, whose stages are too large to be limited in number, limit the
+    // SMs instead (FLUX.1-dev, K = 5: 3/4 of the SMs with all stages 1794 us,
+    // all of them with three stages 1800 us, with all stages 1898 us; K = 8:
+    // 344 and 340 us).
+    double frac = 1.0;
+    if (cb16 && !grouped && !precise && (K == 5 || K == 6) && A.tiles_total >= 8LL * p->dev.sms) {
+        frac = 0.75;
+        A.stages = stages_all;
+        smem = smem_all;
+    }
+    // The gated one-entry epilogue cannot hold two groups of two and keep to its
+    // bytes in flight: a twentieth of the SMs less does it (GB300, groups of
+    // two, [8, 256, 1152], [4, 1024, 1152], [2, 4096, 1152] and [1, 4096, 3072]:
+    // 128.5 -> 125.2, 250 -> 246, 493 -> 486, 658 -> 651 us; groups of one and
+    // three and fp32 gates lose 1 to 4 % by it).
+    if (L.full_step && cb16 && gated && hold && max_nb == 2 && L.gate_dtype == CB_BF16) frac = 0.95;
+    const long long ctas = std::max(1LL, (long long)((double)p->dev.sms * per_sm * frac));
+    const int grid = A.any_scalar ? (int)ctas : (int)std::min<long long>((long long)A.tiles_total + A.n_ragged, ctas);
+    rc = clear_status(L);
+    if (rc != CB_OK) return rc;
+    const cudaStream_t s = (cudaStream_t)L.stream;
+    cudaError_t e = strided   ? cbk::launch_extrapolate_bulk_strided(A, K, cb16, grouped, gated, grid, smem, s)
+                    : precise ? cbk::launch_extrapolate_bulk_precise(A, K, cb16, grouped, gated, grid, smem, s)
+                    : gated   ? cbk::launch_extrapolate_bulk_gated(A, K, cb16, grid, smem, s)
+                              : cbk::launch_extrapolate_bulk(A, K, cb16, grouped, grid, smem, s);
+    return e == cudaSuccess ? CB_OK : cuda_fail(e, "extrapolate launch");
+}
+
 // One skipped-step launch over the window `win` with the fp64 weights w[0..n).
 // With `feats` it is instead a full step's epilogue: a one-entry history (the
 // new features, weight 1) whose members are written, converted, into the ring
@@ -333,38 +560,41 @@ int run_launch(cb_plan* p, const Window& win, const double* w, void* const* outs
     const bool cb16 = (feats ? feat_dtype : p->cache_dtype) == CB_BF16;
     // A full step's epilogue runs its own kernel (unless CB_OPT_KERNEL names
     // one) when its threads keep enough loads in flight: ungated bf16 features
-    // with every tensor in a residual group of three or more branches.
+    // and bf16 hidden states with every tensor in a residual group of three or
+    // more branches.
     // Otherwise the bulk pipeline streams faster (see epilogue.cu).
-    bool epilogue = feats && p->kernel == CB_KERNEL_AUTO && feat_dtype == CB_BF16 && resid;
+    bool epilogue = feats && p->kernel == CB_KERNEL_AUTO && feat_dtype == CB_BF16 && resid &&
+                    resid_dtype == CB_BF16;
     for (int i = 0; epilogue && i < n; ++i) {
         const int g = p->tensors[i].group;
         epilogue = g >= 0 && resid[g] && p->groups[g].size() >= 3 && !(gates && gates[i]);
     }
-    const long long te_bulk = cbk::tile_elems(cb16);
-    const long long te = epilogue ? cbk::epilogue_tile_elems : te_bulk;
     unsigned char* slot = p->cache + (size_t)p->next * p->slot_bytes;
     A.hist_base = feats ? 0ull : (unsigned long long)(uintptr_t)(ch ? ch->hist : p->cache);
     A.copy_out = feats ? 1 : 0;
+    double w_sum = 0.0;
     for (int j = 0; j < CB_MAX_K; ++j) {
         const bool on = j < K;
         A.slot_off[j] = on && !feats ? (long long)win.slot[j] * (long long)p->slot_bytes : 0;
         const float hi = on ? (float)w[j] : 0.0f;
         A.w_hi[j] = hi;
+        w_sum += std::fabs((double)hi);
         A.w_lo[j] = on ? (float)(w[j] - (double)hi) : 0.0f;
         // the fast path's bound, scaled: (K+2) u (1.01) 2^9 |w_hi[j]|, u = 2^-24
         A.w_guard[j] = (float)(std::fabs((double)hi) * (K + 2) * 1.01 * std::ldexp(1.0, -15));
     }
+    A.w_sum = std::nextafterf((float)w_sum, INFINITY);
     A.out_bf16 = out_dtype == CB_BF16;
     A.resid_bf16 = resid_dtype == CB_BF16;
 
     int items = 0, members = 0;
-    long long tiles = 0;
     bool any_out = false, any_resid = false;
-    bool any_gate = false;
+    // items that can be copied in but not stored (or gated) by whole vectors
+    bool strided[cbk::kMaxItems];
     A.gate_bf16 = gate_dtype == CB_BF16;
     auto add_item = [&](const int* mem, int nm, void* res_ptr) {
         const long long numel = p->tensors[mem[0]].numel;
-        bool vec = !res_ptr || aligned(res_ptr, 16);
+        bool vec = !res_ptr || aligned(res_ptr, 16), src = true;
         A.first[items] = (short)members;
         A.i_hidden[items] = (unsigned)p->sh_hidden[mem[0]];
         A.i_row[items] = (unsigned)(p->sh_tokens[mem[0]] * p->sh_hidden[mem[0]]);
@@ -375,11 +605,10 @@ int run_launch(cb_plan* p, const Window& win, const double* w, void* const* outs
             void* o = feats ? slot + p->off[i] : outs ? outs[i] : nullptr;
             const void* g = (res_ptr && gates) ? gates[i] : nullptr;
             A.m_off[members] = feats ? (long long)(uintptr_t)feats[i] : p->off[i];
-            if (feats) vec = vec && aligned(feats[i], 16);
+            if (feats) src = src && aligned(feats[i], 16);
             A.m_out[members] = o;
             A.m_gate[members] = g;
             if (g) {  // vectors of 8 stay inside one gate row
-                any_gate = true;
                 vec = vec && aligned(g, 16) && p->sh_hidden[i] % 8 == 0;
             }
             if (o) {
@@ -388,13 +617,13 @@ int run_launch(cb_plan* p, const Window& win, const double* w, void* const* outs
             }
             ++members;
         }
+        vec = vec && src;
         if (res_ptr) any_resid = true;
         A.nb[items] = (unsigned char)nm;
         A.resid[items] = res_ptr;
         A.vec_ok[items] = vec ? 1 : 0;
+        strided[items] = !vec && src;
         A.numel[items] = numel;
-        A.tile_begin[items] = (int)tiles;
-        tiles += (numel + te - 1) / te;
         ++items;
     };
     std::vector<char> in_group(n, 0);
@@ -406,10 +635,7 @@ int run_launch(cb_plan* p, const Window& win, const double* w, void* const* outs
             }
     for (int i = 0; i < n; ++i)
         if (!in_group[i] && (feats || (outs && outs[i]))) add_item(&i, 1, nullptr);
-    if (tiles > 0x7FFFFFFFLL) return CB_ERR_LIMIT;
-    A.tile_begin[items] = (int)tiles;
     A.n_items = items;
-    A.tiles_total = (int)tiles;
     // a full step's slot write is a conversion, not arithmetic
     A.precise = (any_out && !feats && out_dtype == CB_FP32) || (any_resid && resid_dtype == CB_FP32);
     if (items == 0) return CB_OK;  // nothing requested
@@ -418,131 +644,28 @@ int run_launch(cb_plan* p, const Window& win, const double* w, void* const* outs
     A.status = ch ? ch->status : p->status_word();
     A.withhold_first = p->withhold_first;
     A.stages = 0;
-    A.stage_chunks = K;
-    A.stage_x = 0;
+    A.stage_x_bytes = 0;
     A.stage_gate_bytes = 0;
+    A.n_ragged = A.any_scalar = 0;
 
     rc = ensure_device(p);
     if (rc != CB_OK) return rc;
-    auto clear_status = [&]() {
-        if (!ch) return clear_status_once(p, stream);
-        const int r = clear_word(ch->status, stream);
-        ch->launched = r == CB_OK;
-        return r;
-    };
-    auto launch_direct = [&]() {
-        int grid = 0;
-        int r = extrap_grid(p, K, cb16, (int)tiles, &grid);
-        if (r != CB_OK) return r;
-        r = clear_status();
-        if (r != CB_OK) return r;
-        cudaError_t e = any_gate ? cbk::launch_extrapolate_gated(A, K, cb16, grid, (cudaStream_t)stream)
-                                 : cbk::launch_extrapolate(A, K, cb16, grid, (cudaStream_t)stream);
-        if (e != cudaSuccess) return cuda_fail(e, "extrapolate launch");
-        return (int)CB_OK;
-    };
-    if (epilogue) {
-        int& occ = p->dev.occ_epilogue;
-        if (occ == 0) {
-            cudaError_t e = cbk::epilogue_blocks_per_sm(&occ);
-            if (e != cudaSuccess || occ <= 0) {
-                occ = 0;
-                return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "occupancy");
-            }
-        }
-        const long long ctas = (long long)p->dev.sms * occ;
-        const int grid = (int)(tiles < ctas ? tiles : ctas);
-        rc = clear_status();
-        if (rc != CB_OK) return rc;
-        cudaError_t e = cbk::launch_epilogue(A, grid, (cudaStream_t)stream);
-        if (e != cudaSuccess) return cuda_fail(e, "epilogue launch");
-        return CB_OK;
-    }
-    if (p->kernel == CB_KERNEL_DIRECT) return launch_direct();
-    // bf16 hidden states travel through shared memory with the last member of
-    // their group; the pipeline must hold a whole group plus one stage ahead
-    int max_nb = 1;
-    for (int i = 0; i < items; ++i)
-        if (A.nb[i] > max_nb) max_nb = A.nb[i];
-    A.stage_x = any_resid && A.resid_bf16 ? 1 : 0;
-    A.stage_chunks = K + A.stage_x;
-    // gate rows travel with their member when every gated tile touches at
-    // most two batches (a batch holds a tile or more) and two rows are small
-    A.stage_gate_bytes = 0;
-    if (any_gate) {
-        const size_t gs = esize(gate_dtype);
-        size_t need = 0;
-        bool fits = true;
-        for (int i = 0; i < items; ++i) {
-            bool gated_item = false;
-            for (int m = 0; m < A.nb[i]; ++m) gated_item = gated_item || A.m_gate[A.first[i] + m];
-            if (!gated_item || !A.vec_ok[i]) continue;
-            fits = fits && (long long)A.i_row[i] >= te_bulk;
-            need = std::max(need, 2 * (size_t)A.i_hidden[i] * gs);
-        }
-        if (fits && need <= kMaxStagedGateBytes) A.stage_gate_bytes = (unsigned)((need + 127) / 128 * 128);
-    }
-    // the grouped kernel (hidden-state bookkeeping) for gates, hidden states or multi-member items
-    bool grouped = any_gate;
-    for (int i = 0; i < items; ++i) grouped = grouped || A.resid[i] != nullptr || A.nb[i] > 1;
-    size_t smem = 0;
-    int per_sm = 1;
-    rc = bulk_config(p, K, cb16, grouped, A.stage_chunks, A.stage_gate_bytes, any_gate, max_nb + 1, &A.stages,
-                     &smem, &per_sm);
+    Launch L{p, K, cb16, feats != nullptr, res, gate_dtype, stream, ch};
+    if (p->kernel == CB_KERNEL_DIRECT) return launch_direct(L, A);
+    auto aligned_items = [&](cbk::ExtrapArgs& B) { return epilogue ? launch_epilogue(L, B) : launch_bulk(L, B, false); };
+    int n_strided = 0;
+    for (int i = 0; i < items; ++i) n_strided += strided[i] ? 1 : 0;
+    if (n_strided == 0) return aligned_items(A);
+    if (n_strided == items) return launch_bulk(L, A, true);
+    // some of each: a launch for either
+    if (!p->eargs2) p->eargs2.reset(new (std::nothrow) cbk::ExtrapArgs());
+    if (!p->eargs2) return CB_ERR_LIMIT;
+    cbk::ExtrapArgs& B = *p->eargs2;
+    take_items(A, strided, true, B);
+    rc = launch_bulk(L, B, true);
     if (rc != CB_OK) return rc;
-    if (A.stages < max_nb + 1) return launch_direct();  // too deep for shared memory
-    const int stages_all = A.stages;
-    const size_t smem_all = smem;
-    // Bytes in flight. HBM serves a mix of reads and writes best when no more is
-    // asked of it than covers its latency; beyond that reads and writes turn
-    // the bus around more often. GB300, DiT-XL/2 256^2 shapes, every SM, KB in
-    // flight per SM (all that fits -> here): predictions with K = 1 100.0 ->
-    // 83.8 us (48), K = 2 136 -> 120 (64), K = 3 169 -> 151 (120), K = 4 206 ->
-    // 188 (128); full-step epilogue from fp32 features 176 -> 159 (100). The
-    // more is read per byte written, the flatter the optimum and the higher.
-    // Launches that hold a group's stages keep two groups' worth; those with
-    // K >= 2 are bound by their consumers and any depth serves them.
-    if (!grouped || K == 1) {
-        double rd = 0, wr = 0, units = 0;
-        for (int i = 0; i < items; ++i) {
-            const double e = (double)A.numel[i], x = A.resid[i] ? (double)res : 0.0;
-            rd += e * (A.nb[i] * K * (cb16 ? 2.0 : 4.0) + x);
-            units += e * A.nb[i];
-            wr += e * x;
-            for (int m = 0; m < A.nb[i]; ++m)
-                if (A.m_out[A.first[i] + m]) wr += e * (A.out_bf16 ? 2.0 : 4.0);
-        }
-        const double ratio = rd / wr, kb = grouped ? 96 : ratio < 1.25 ? 48 : ratio < 2.5 ? 76 : 120;
-        const double unit = rd / units * te_bulk;
-        const int most = (int)(kb * 1024.0 / unit / per_sm + 0.5);
-        const int least = std::max(grouped ? 2 * max_nb : 2, per_sm == 1 ? 3 : 2);
-        // bf16 features leave the consumers the bound: those keep every stage
-        if (!(grouped && cb16)) {
-            const int keep = std::max(most, least);
-            if (keep < A.stages) {
-                A.stages = keep;
-                smem = cbk::bulk_smem_bytes(A.stage_chunks, A.stage_gate_bytes, keep);
-            }
-        }
-    }
-    // Persistent grid: every SM, except that bf16 prediction-only launches with
-    // K >= 5, whose stages are too large to be limited in number, limit the
-    // SMs instead (FLUX.1-dev, 3/4 of the SMs with all stages 1788 us, all of
-    // them with three stages 1800 us, with all stages 1898 us).
-    double frac = 1.0;
-    if (cb16 && !grouped && K >= 5 && tiles >= 8LL * p->dev.sms) {
-        frac = 0.75;
-        A.stages = stages_all;
-        smem = smem_all;
-    }
-    const long long ctas = std::max(1LL, (long long)((double)p->dev.sms * per_sm * frac));
-    const int grid = (int)(tiles < ctas ? tiles : ctas);
-    rc = clear_status();
-    if (rc != CB_OK) return rc;
-    cudaError_t e = any_gate ? cbk::launch_extrapolate_bulk_gated(A, K, cb16, grid, smem, (cudaStream_t)stream)
-                             : cbk::launch_extrapolate_bulk(A, K, cb16, grouped, grid, smem, (cudaStream_t)stream);
-    if (e != cudaSuccess) return cuda_fail(e, "extrapolate launch");
-    return CB_OK;
+    take_items(A, strided, false, B);
+    return aligned_items(B);
 }
 
 }  // namespace

@@ -1,0 +1,152 @@
+"""Tiles and items at the edges of the bulk kernel's paths (GPU): ragged last
+tiles around every tile size, outputs, hidden states and gates off the 16-byte
+grid (alone and beside aligned items), and compensated sums at the ends of the
+number range."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as orc
+from paper_2608_23429_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cb():
+    from paper_2608_23429_gb300 import chebboost
+    return chebboost
+
+
+@pytest.fixture(scope="module")
+def H():
+    import gpu_harness
+    return gpu_harness
+
+
+def _workload(K, cache):
+    """Lone tensors of one element around the tile sizes 2048, 2816, 4096 and
+    4864, and groups of odd and even channel counts."""
+    T = workloads.TensorSpec
+    tensors = [T(0, b, (2, 37, 77), 0) for b in range(3)] + [T(1, b, (3, 41, 136), 1) for b in range(2)]
+    tensors += [T(2, 0, (1, 1, 1), 2), T(3, 0, (2, 2816, 1), 3)]
+    tensors += [T(4 + i, 0, (1, 1, n), -1)
+                for i, n in enumerate([7, 2047, 2049, 2815, 2816, 4095, 4097, 4863, 4864, 9733])]
+    return workloads.Workload(name="edges", tensors=tensors, K=K, cache_dtype=cache, T=0, r=0, t_min=0.0, t_max=999.0,
+                              timesteps=[], degree=6, noise=0.1, seed=77)
+
+
+def _shifted(shape, dtype, off):
+    """A view `off` elements into its buffer, and the buffer (filled with ones)."""
+    n = int(np.prod(shape))
+    buf = torch.ones(n + off + 9, dtype=dtype, device="cuda")
+    return buf[off:off + n].view(shape), buf
+
+
+@pytest.mark.parametrize("shift", ["none", "some", "all"])
+@pytest.mark.parametrize("K,cache,io", [(1, "bf16", "fp32"), (2, "bf16", "bf16"), (2, "fp32", "fp32"),
+                                        (3, "bf16", "fp32"), (4, "fp32", "bf16"), (5, "bf16", "bf16"),
+                                        (8, "bf16", "fp32"), (8, "fp32", "fp32")])
+def test_ragged_tiles_and_off_grid_items(cb, H, K, cache, io, shift):
+    w = _workload(K, cache)
+    nodes = [990.0 - 37.0 * k for k in range(K)]
+    walk = H.Walk(w, node_t=nodes)
+    cb.cb_plan_set_shapes(walk.plan, [s.shape for s in w.tensors])
+    for k, t in enumerate(nodes):
+        walk.push(t, k)
+    dt, target = H.TORCH[io], nodes[-1] - 20.0
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    gates = [(0.5 * torch.randn(s.shape[0], s.shape[2], generator=gen, device="cuda")).to(dt) if i % 3 != 1 else None
+             for i, s in enumerate(w.tensors)]
+    for gated in (False, True):
+        off = [0 if shift == "none" or (shift == "some" and i % 2) else 1 + i % 7 for i in range(len(w.tensors))]
+        outs, bufs = zip(*[_shifted(s.shape, dt, o) for s, o in zip(w.tensors, off)])
+        resid, rbufs, rh = [], [], []
+        for g in range(walk.n_groups):
+            x, b = _shifted(w.group_shape(g), dt, off[g])
+            x.copy_(workloads.hidden_state(w, g, "cuda", dt, salt=9))
+            resid.append(x)
+            rbufs.append(b)
+            rh.append(H.host(x))
+        if gated:
+            cb.cb_extrapolate_gated(walk.plan, target, outs, H.CB[io], resid, H.CB[io], gates, H.CB[io])
+        else:
+            cb.cb_extrapolate(walk.plan, target, outs, H.CB[io], resid, H.CB[io])
+        torch.cuda.synchronize()
+        assert cb.cb_plan_device_status(walk.plan) == 0
+        G = [None if g is None else H.expand_gate(g, s.shape) for g, s in zip(gates, w.tensors)] if gated else None
+        so, sr, _ = walk.expected_and_compare(target, outs, resid, rh, out_dtype=io, resid_dtype=io, G=G)
+        assert so["bad"] == 0 and sr["bad"] == 0, (gated, so, sr)
+        for buf, o, s in list(zip(bufs, off, w.tensors)) + [(b, off[g], next(t for t in w.tensors if t.group == g))
+                                                           for g, b in enumerate(rbufs)]:
+            assert torch.all(buf[:o] == 1) and torch.all(buf[o + s.numel:] == 1)  # nothing beside the tensor
+    walk.close()
+
+
+@pytest.mark.parametrize("kernel", ["bulk", "direct"])
+@pytest.mark.parametrize("cache", ["bf16", "fp32"])
+@pytest.mark.parametrize("n", [9728, 1234])
+def test_compensated_sums_at_the_ends_of_the_range(cb, H, cache, kernel, n):
+    """Features up to the largest finite value, where the sum's anchor would
+    overflow, and infinities and NaN: the newest entry alone (weights 0, 0, 1)
+    comes back exactly, and only elements that hold no number give none."""
+    w = workloads.Workload(name="range", tensors=[workloads.TensorSpec(0, 0, (1, 1, n), 0)], K=3, cache_dtype=cache, T=0,
+                           r=0, t_min=0.0, t_max=999.0, timesteps=[], degree=3, noise=0.1, seed=3)
+    walk = H.Walk(w, node_t=[900.0, 800.0, 700.0], kernel=kernel)
+    dt = H.TORCH[cache]
+    feats = [workloads.trajectory(w, 0, t, k, "cuda", out_dtype=dt) for k, t in enumerate(walk.node_t)]
+    big, flat = float(torch.finfo(dt).max), feats[2].reshape(-1)
+    for i, v in enumerate([big, -big, big / 8, float(torch.finfo(dt).tiny), 0.0, -0.0]):
+        flat[100 * i + 3] = v
+    flat[901], flat[902], flat[n - 1] = float("inf"), float("nan"), -big
+    for t, f in zip(walk.node_t, feats):
+        cb.cb_cache_push(walk.plan, [f], H.CB[cache], t)
+    out = torch.empty(n, dtype=torch.float32, device="cuda")
+    x = torch.zeros(n, dtype=torch.float32, device="cuda")
+    cb.cb_extrapolate_weights(walk.plan, np.array([0.0, 0.0, 1.0]), [out], cb.CB_FP32, [x], cb.CB_FP32)
+    torch.cuda.synchronize()
+    want = flat.float()
+    fine = torch.isfinite(want)
+    assert torch.equal(out[fine], want[fine]) and torch.equal(x[fine], want[fine])
+    assert not torch.isfinite(out[~fine]).any() and not torch.isfinite(x[~fine]).any()
+    walk.close()
+
+
+@pytest.mark.parametrize("src", ["bf16", "fp32"])
+@pytest.mark.parametrize("io", ["bf16", "fp32"])
+def test_full_step_beside_off_grid_hidden_states(cb, H, src, io):
+    """A full step whose hidden states lie partly off the 16-byte grid writes
+    the cache write's bytes and the oracle's hidden states."""
+    w = _workload(3, "bf16")
+    nodes = [900.0, 800.0, 700.0]
+    a, b = H.Walk(w, node_t=nodes), H.Walk(w, node_t=nodes)
+    dt = H.TORCH[io]
+    offs, slot = H.slot_layout([s.numel for s in w.tensors], 2)
+    for k, t in enumerate(nodes):
+        feats = [workloads.trajectory(w, i, t, k, "cuda", out_dtype=H.TORCH[src]) for i in range(len(w.tensors))]
+        resid = []
+        for g in range(a.n_groups):
+            x, _ = _shifted(w.group_shape(g), dt, (g + k) % 2)
+            x.copy_(workloads.hidden_state(w, g, "cuda", dt, salt=k))
+            resid.append(x)
+        rh = [H.host(x) for x in resid]
+        cb.cb_cache_push_residual(a.plan, feats, H.CB[src], t, resid, H.CB[io])
+        cb.cb_cache_push(b.plan, feats, H.CB[src], t)
+        torch.cuda.synchronize()
+        assert cb.cb_plan_device_status(a.plan) == 0
+        for i, s in enumerate(w.tensors):
+            lo = k * slot + offs[i]
+            assert torch.equal(a.cache[lo:lo + 2 * s.numel], b.cache[lo:lo + 2 * s.numel]), (k, i)
+        for g in range(a.n_groups):
+            F = [[H.host(feats[i])] for i, s in enumerate(w.tensors) if s.group == g]
+            _, r64 = orc.extrapolate(F, [1.0], H.ORC[src], None, X=rh[g], x_dtype=H.ORC[io], resid_dtype=orc.FP64)
+            f64 = [H.bf16_to_f64(f[0]) if src == "bf16" else f[0].astype(np.float64) for f in F]
+            x64 = H.bf16_to_f64(rh[g]) if io == "bf16" else rh[g].astype(np.float64)
+            if io == "bf16":
+                st = H.compare_bf16(H.host(resid[g]), orc.convert(r64, orc.FP64, orc.BF16), r64,
+                                    np.abs(np.array(f64)).sum(0) + np.abs(x64))
+            else:
+                st = H.compare_fp32(H.host(resid[g]), r64, float(np.max(np.abs(f64))))
+            assert st["bad"] == 0, (k, g, st)
+    a.close()
+    b.close()
