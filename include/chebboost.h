@@ -207,9 +207,9 @@ int cb_extrapolate_ring(cb_plan* plan, const double* slot_t, int head, double t_
  *       as cb_extrapolate_ring. Every slot must hold an entry.
  * status: host pointer (may be NULL). It receives the launch's device status
  *       word (CB_DEV_* codes, 0 = none) once the stream has reached the end
- *       of this call. The value arrives by an asynchronous device-to-host
- *       copy when *status is pinned memory. With ordinary memory the copy,
- *       and thus this call, waits for the launch to finish.
+ *       of this call. The device writes it when *status is pinned memory.
+ *       With ordinary memory it is copied, and this call waits for the launch
+ *       to finish.
  *
  * Allocation: the call allocates no device memory and no pinned host memory.
  * Its status block is a file-scope device array of CB_STATUS_BYTES (256) bytes. Every GPU that
@@ -221,10 +221,10 @@ int cb_extrapolate_ring(cb_plan* plan, const double* slot_t, int head, double t_
  * Set-up: the first call on each device looks up the block's device address
  * there (cudaGetSymbolAddress, with that device current). Make that first call
  * before any stream capture begins.
- * Sharing: every call on a device uses the same word. Each launch clears it
- * first on its own stream. Calls that overlap on the GPU (different streams,
- * no ordering between them) race on it: one may clear or read another's
- * code. Their outputs are unaffected.
+ * Sharing: every call on a device that asks for its status uses the same word,
+ * which is cleared as its value is handed over. Such calls that overlap on the
+ * GPU (different streams, no ordering between them) race on it: one may clear
+ * or read another's code. Their outputs are unaffected.
  * Errors: as cb_extrapolate_ring (CB_ERR_UNBOUND excepted), plus CB_ERR_ALIGN
  * for hist and CB_ERR_CUDA when the status block cannot be reached. A
  * CB_ERR_CUDA from the status read-back comes after the launch was enqueued. */

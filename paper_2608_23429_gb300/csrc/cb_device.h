@@ -162,5 +162,7 @@ cudaError_t push_blocks_per_sm(bool src_bf16, bool dst_bf16, int* blocks);
 // current device. The first call per device looks the address up.
 constexpr int kMaxStatusDevices = 64;
 cudaError_t noalloc_status_word(int device, int** word);
+// Hands the word over to *status (memory the device can write) and clears it.
+cudaError_t take_status(int* word, int* status, cudaStream_t s);
 
 }  // namespace cbk

@@ -294,19 +294,13 @@ int clear_status_once(cb_plan* p, void* stream) {
 }
 
 // A history buffer given with the call instead of the bound arena, and the
-// status word its launch records into (cb_extrapolate_noalloc). `launched` is
-// set once the word has been cleared for a launch.
+// status word its launches record into (cb_extrapolate_noalloc; null: none).
+// `launched` is set once a launch is under way.
 struct CallerHistory {
     const unsigned char* hist;
     int* status;
     bool launched;
 };
-
-// Zero a status word that every call shares, on the launch's stream.
-int clear_word(int* word, void* stream) {
-    cudaError_t e = cudaMemsetAsync(word, 0, sizeof(int), (cudaStream_t)stream);
-    return e == cudaSuccess ? CB_OK : cuda_fail(e, "cudaMemsetAsync");
-}
 
 // What the launches of one call share.
 struct Launch {
@@ -318,15 +312,12 @@ struct Launch {
     cb_dtype gate_dtype;
     void* stream;
     CallerHistory* ch;
-    bool cleared = false;
 };
 
 int clear_status(Launch& L) {
     if (!L.ch) return clear_status_once(L.p, L.stream);
-    if (L.cleared) return CB_OK;
-    const int r = clear_word(L.ch->status, L.stream);
-    L.ch->launched = L.cleared = r == CB_OK;
-    return r;
+    L.ch->launched = true;  // that word is zero (static_status.cu)
+    return CB_OK;
 }
 
 // Cut the items into tiles of te elements, numbered across items. `split` (the
@@ -882,17 +873,26 @@ int cb_extrapolate_noalloc(cb_plan* p, const void* hist, size_t hist_bytes, cons
     int* word = nullptr;
     e = cbk::noalloc_status_word(dev, &word);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress");
-    CallerHistory ch{static_cast<const unsigned char*>(hist), word, false};
+    // Only launches whose status is asked for record into the word, and handing
+    // it over clears it, so that it needs no clearing before a launch.
+    CallerHistory ch{static_cast<const unsigned char*>(hist), status ? word : nullptr, false};
     rc = run_launch(p, win, w, outs, out_dtype, resid, resid_dtype, stream, nullptr, CB_BF16, nullptr, CB_BF16, &ch);
-    if (rc != CB_OK) return rc;
-    if (status) {
-        if (!ch.launched) {  // nothing was requested, so nothing ran
-            *status = 0;
-            return CB_OK;
-        }
-        e = cudaMemcpyAsync(status, word, sizeof(int), cudaMemcpyDeviceToHost, (cudaStream_t)stream);
-        if (e != cudaSuccess) return cuda_fail(e, "status read-back");
+    if (rc != CB_OK || !status) return rc;
+    if (!ch.launched) {  // nothing was requested, so nothing ran
+        *status = 0;
+        return CB_OK;
     }
+    cudaPointerAttributes at{};
+    const bool pinned = cudaPointerGetAttributes(&at, status) == cudaSuccess && at.type == cudaMemoryTypeHost &&
+                        at.devicePointer != nullptr;
+    if (pinned) {
+        e = cbk::take_status(word, static_cast<int*>(at.devicePointer), (cudaStream_t)stream);
+    } else {
+        (void)cudaGetLastError();  // a pointer the runtime does not know is ordinary memory
+        e = cudaMemcpyAsync(status, word, sizeof(int), cudaMemcpyDeviceToHost, (cudaStream_t)stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(word, 0, sizeof(int), (cudaStream_t)stream);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "status read-back");
     return CB_OK;
 }
 

@@ -27,9 +27,16 @@ namespace {
 std::mutex g_mu;
 int* g_addr[cbk::kMaxStatusDevices] = {};
 
+__global__ void take_status_kernel(int* word, int* status) { *status = atomicExch(word, 0); }
+
 }  // namespace
 
 namespace cbk {
+
+cudaError_t take_status(int* word, int* status, cudaStream_t s) {
+    take_status_kernel<<<1, 1, 0, s>>>(word, status);
+    return cudaGetLastError();
+}
 
 cudaError_t noalloc_status_word(int device, int** word) {
     if (device < 0 || device >= kMaxStatusDevices) return cudaErrorInvalidDevice;

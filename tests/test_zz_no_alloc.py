@@ -105,3 +105,33 @@ def test_noalloc_matches_ring_on_two_calls(cb, H):
         assert e.value.status == code
     cb.cb_plan_destroy(plan)
     walk.close()
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+def test_noalloc_status_is_handed_over_once(cb, H, pinned):
+    """A launch whose wait runs out (its first copies are withheld) reports its
+    code, in pinned and in ordinary memory, and the next launch reports none,
+    also after one that nobody asked about."""
+    w = _workload()
+    plan = cb.cb_plan_create(NODES, K, [(t.layer, t.branch, t.numel, t.group) for t in w.tensors], H.CB["bf16"], w.t_min,
+                             w.t_max)
+    nbytes = cb.cb_plan_cache_bytes(plan) - cb.CB_STATUS_BYTES
+    hist = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
+    outs = [torch.empty(s.shape, dtype=torch.bfloat16, device="cuda") for s in w.tensors]
+    cb.cb_plan_set_option(plan, cb.CB_OPT_WAIT_NS, 1000000)
+
+    def call(withhold, asked=True):
+        status = torch.full((1,), -1, dtype=torch.int32)
+        status = status.pin_memory() if pinned else status
+        cb.cb_plan_set_option(plan, cb.CB_OPT_TEST_WITHHOLD, int(withhold))
+        cb.cb_extrapolate_noalloc(plan, hist, nbytes, NODES[:K], 0, 820.0, outs, cb.CB_BF16,
+                                  status=status if asked else None)
+        torch.cuda.synchronize()
+        return int(status[0])
+
+    assert call(False) == 0
+    assert call(True) & cb.CB_DEV_CONSUMER_TIMEOUT
+    assert call(False) == 0
+    assert call(True, asked=False) == -1
+    assert call(False) == 0
+    cb.cb_plan_destroy(plan)
