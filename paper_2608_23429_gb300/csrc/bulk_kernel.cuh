@@ -205,6 +205,24 @@ __device__ __forceinline__ uint2 ragged_pair(const unsigned char* p, int i, int 
     return w;
 }
 
+// Four pairs of elements p[at(q, 0)], p[at(q, 1)]; 0 where at() is negative.
+template <typename At>
+__device__ __forceinline__ void read_pairs(const void* p, bool bf16, float (&x)[8], At at) {
+    if (bf16) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const long long e = at(i >> 1, i & 1);
+            x[i] = e >= 0 ? __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(p)[e] << 16) : 0.0f;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const long long e = at(i >> 1, i & 1);
+            x[i] = e >= 0 ? reinterpret_cast<const float*>(p)[e] : 0.0f;
+        }
+    }
+}
+
 // The consumers of launches with fp32 predictions or hidden states: every
 // element takes the compensated sum (sum_vec), so nothing is recomputed and
 // each stage goes back to the producer as soon as its values, and the hidden
@@ -257,16 +275,27 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
         for (int v = 0; v < U; ++v) ev[v] = e0 + at(v);
         if (gated) gate_offsets<U>(A, it, e0, ev, gi);
     }
+    // ragged: of the pairs' first elements, and whether the second one lies in
+    // the next token of the same batch, hidden channels back
+    unsigned gq[U][4], back = 0u;
+    if constexpr (GATED && RAGGED) {
+        if (gated)
+#pragma unroll
+            for (int v = 0; v < U; ++v)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    bool b;
+                    gate_offset_pair(A, it, e0 + (pair_at(v, q) < n ? pair_at(v, q) : 0), gq[v][q], b);
+                    back |= b ? 1u << (4 * v + q) : 0u;
+                }
+    }
     Acc<U> acc;
     Finite fin;
     if (GROUPED && RAGGED && resid != nullptr)  // not staged: asked for before the wait for the stage
         resid_begin<U>(acc, [&](int v, float (&x)[8]) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int i = pair_at(v, q);
-                x[2 * q] = i < n ? load_elem(resid, A.resid_bf16, e0 + i) : 0.0f;
-                x[2 * q + 1] = i + 1 < n ? load_elem(resid, A.resid_bf16, e0 + i + 1) : 0.0f;
-            }
+            read_pairs(resid, A.resid_bf16, x, [&](int q, int e) {
+                return pair_at(v, q) + e < n ? e0 + pair_at(v, q) + e : -1ll;
+            });
         });
 #pragma unroll 1
     for (int m = 0; m < nb; ++m) {
@@ -284,15 +313,10 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
 #pragma unroll
                 for (int e = 0; e < 8; ++e) g[v][e] = 1.0f;
                 if (RAGGED && gp != nullptr)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int i = pair_at(v, q);
-                        if (i >= n) continue;
-                        unsigned g0, g1;
-                        gate_offset_pair(A, it, e0 + i, g0, g1);
-                        g[v][2 * q] = load_elem(gp, A.gate_bf16, g0);
-                        if (i + 1 < n) g[v][2 * q + 1] = load_elem(gp, A.gate_bf16, g1);
-                    }
+                    read_pairs(gp, A.gate_bf16, g[v], [&](int q, int e) {
+                        const long long at = gq[v][q] + e - (e && (back >> (4 * v + q) & 1u) ? A.i_hidden[it] : 0u);
+                        return pair_at(v, q) + e < n ? at : -1ll;
+                    });
             }
         }
         const uint32_t stage = cur.stage;

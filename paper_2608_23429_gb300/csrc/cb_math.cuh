@@ -125,6 +125,18 @@ __device__ __forceinline__ uint16_t bf16_of_pair(float hi, float lo) {
     return bf16_bits(hi);
 }
 
+// hi + lo (hi = fl(hi + lo), finite) rounded to odd: of the two fp32 values about
+// it the one with an odd last bit, unless it is exact. Rounding that to nearest
+// bf16 gives what rounding hi + lo gives (Boldo & Melquiond, "Emulation of a
+// FMA and correctly rounded sums: proved algorithms using rounding to odd",
+// IEEE Trans. Comput. 57(4), 2008).
+__device__ __forceinline__ float odd_of_pair(float hi, float lo) {
+    const uint32_t b = __float_as_uint(hi);
+    const bool inexact = lo != 0.0f && (b & 1u) == 0u && (b & 0x7F800000u) != 0x7F800000u;
+    const uint32_t step = 1u | (uint32_t)((int)(b ^ __float_as_uint(lo)) >> 31);  // away from zero 1, towards it -1
+    return __uint_as_float(inexact ? b + step : b);
+}
+
 // Start of history entry j of the member at byte offset moff.
 __device__ __forceinline__ const unsigned char* hist_ptr(const ExtrapArgs& A, int j, long long moff) {
     return reinterpret_cast<const unsigned char*>(A.hist_base + (unsigned long long)A.slot_off[j] +
@@ -293,7 +305,7 @@ using RawVecs = uint4[UV][K][CB16 ? 1 : 2];
 // elements of a vector: fp32 in o[0..7], or bf16 in o[0..3].
 __device__ __forceinline__ void put_pair(uint32_t (&o)[8], bool bf16, int q, float2 hi, float2 lo) {
     if (bf16) {
-        o[q] = (uint32_t)bf16_of_pair(hi.x, lo.x) | ((uint32_t)bf16_of_pair(hi.y, lo.y) << 16);
+        o[q] = pack_bf16x2(odd_of_pair(hi.x, lo.x), odd_of_pair(hi.y, lo.y));
     } else {
         o[2 * q] = __float_as_uint(hi.x);
         o[2 * q + 1] = __float_as_uint(hi.y);
@@ -807,15 +819,15 @@ __device__ __forceinline__ void gate_offsets(const ExtrapArgs& A, int it, long l
     }
 }
 
-// Gate offsets of the elements e and e + 1 (32-bit, as above; e + 1 may lie in
-// the next channel row, token or batch). The item has a shape.
-__device__ __forceinline__ void gate_offset_pair(const ExtrapArgs& A, int it, long long e, unsigned& g0, unsigned& g1) {
+// Gate offset g0 of element e (32-bit, as above), of an item with a shape; that
+// of e + 1 is g0 + 1, less the hidden size where it begins the batch's next
+// token (`back`).
+__device__ __forceinline__ void gate_offset_pair(const ExtrapArgs& A, int it, long long e, unsigned& g0, bool& back) {
     const unsigned row = A.i_row[it], H = A.i_hidden[it], ue = (unsigned)e;
     const unsigned b = div_magic(ue, A.i_row_magic[it]), r = ue - b * row;
     const unsigned h = r - div_magic(r, A.i_hidden_magic[it]) * H;
     g0 = b * H + h;
-    g1 = g0 + 1;
-    if (h + 1 == H && r + 1 < row) g1 -= H;  // the next token of the same batch
+    back = h + 1 == H && r + 1 < row;
 }
 
 // The 8 gate values of member mi for each of UV vectors (1 without a gate).
