@@ -614,6 +614,7 @@ __global__ void __launch_bounds__(Shape<CB16, K, GROUPED, GATED, PRECISE>::threa
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    after_previous();
 
     // offset of the gate rows in a stage (a grouped launch has hidden states)
     const uint32_t gates_at =

@@ -79,6 +79,7 @@ __device__ __forceinline__ void epilogue_vector(const ExtrapArgs& A, int it, con
 template <bool CB16, bool GATED>
 __global__ void __launch_bounds__(kThreads, kEpilogueCtasPerSm) epilogue_kernel(const __grid_constant__ ExtrapArgs A) {
     constexpr long long TE = epilogue_tile_elems;
+    after_previous();
     int it = 0;
     for (int tile = blockIdx.x; tile < A.tiles_total; tile += gridDim.x) {
         while (tile >= A.tile_begin[it + 1]) ++it;  // tiles only grow: walk forward
@@ -101,8 +102,7 @@ __global__ void __launch_bounds__(kThreads, kEpilogueCtasPerSm) epilogue_kernel(
 
 // Only the case the host runs here is instantiated: bf16 features, no gates.
 cudaError_t launch_epilogue(const ExtrapArgs& a, int grid, cudaStream_t s) {
-    epilogue_kernel<true, false><<<grid, kThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_overlapped(epilogue_kernel<true, false>, grid, kThreads, 0, s, a);
 }
 
 cudaError_t epilogue_blocks_per_sm(int* blocks) {

@@ -9,15 +9,15 @@ namespace {
 template <int K, bool CB16, bool ONE>
 cudaError_t launch_kk(const ExtrapArgs& a, bool grouped, int grid, size_t smem, cudaStream_t s) {
     if (grouped)
-        extrapolate_bulk_kernel<K, CB16, true, false, ONE><<<grid, Shape<CB16, K, true, false, false>::threads, smem, s>>>(a);
-    else
-        extrapolate_bulk_kernel<K, CB16, false, false, ONE><<<grid, Shape<CB16, K, false, false, false>::threads, smem, s>>>(a);
-    return cudaGetLastError();
+        return launch_overlapped(extrapolate_bulk_kernel<K, CB16, true, false, ONE>, grid,
+                                 Shape<CB16, K, true, false, false>::threads, smem, s, a);
+    return launch_overlapped(extrapolate_bulk_kernel<K, CB16, false, false, ONE>, grid,
+                             Shape<CB16, K, false, false, false>::threads, smem, s, a);
 }
 
-// The full-step epilogue from bf16 features (a copy_out launch) runs the ONE instantiations. From fp32 features
-// the general path measured faster on GB300 (FLUX 95.6 % against 89.0 % of the
-// copy peak), so those launches keep it.
+// The full-step epilogue from bf16 features (a copy_out launch) runs the ONE
+// instantiations. From fp32 features the general path measured faster on GB300
+// (FLUX 95.6 % against 89.0 % of the copy peak), so those launches keep it.
 template <int K, bool CB16>
 cudaError_t launch_k(const ExtrapArgs& a, bool grouped, int grid, size_t smem, cudaStream_t s) {
     if constexpr (K == 1 && CB16)

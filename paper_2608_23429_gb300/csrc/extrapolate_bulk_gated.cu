@@ -5,18 +5,15 @@
 namespace cbk {
 namespace {
 
-// The full-step epilogue from bf16 features (a copy_out launch) runs the ONE instantiation; from fp32 features
-// the general path (see extrapolate_bulk.cu).
+// The full-step epilogue from bf16 features (a copy_out launch) runs the ONE
+// instantiation; from fp32 features the general path (see extrapolate_bulk.cu).
 template <int K, bool CB16>
 cudaError_t launch_gk(const ExtrapArgs& a, int grid, size_t smem, cudaStream_t s) {
-    if constexpr (K == 1 && CB16) {
-        if (a.copy_out) {
-            extrapolate_bulk_kernel<K, CB16, true, true, true><<<grid, Shape<CB16, K, true, true, false>::threads, smem, s>>>(a);
-            return cudaGetLastError();
-        }
-    }
-    extrapolate_bulk_kernel<K, CB16, true, true><<<grid, Shape<CB16, K, true, true, false>::threads, smem, s>>>(a);
-    return cudaGetLastError();
+    constexpr int threads = Shape<CB16, K, true, true, false>::threads;
+    if constexpr (K == 1 && CB16)
+        if (a.copy_out)
+            return launch_overlapped(extrapolate_bulk_kernel<K, CB16, true, true, true>, grid, threads, smem, s, a);
+    return launch_overlapped(extrapolate_bulk_kernel<K, CB16, true, true>, grid, threads, smem, s, a);
 }
 
 template <int K, bool CB16>

@@ -185,19 +185,22 @@ int bulk_config(cb_plan* p, int K, bool cb16, bool gated, bool precise, bool str
     return CB_OK;
 }
 
-int push_grid(cb_plan* p, bool sb, bool db, int tiles, int* grid) {
+// The cache write's grid, and shared memory that it does not use but that keeps
+// an overlapping launch's blocks from crowding on some SMs.
+int push_grid(cb_plan* p, bool sb, bool db, int tiles, int* grid, size_t* smem) {
+    // fewer concurrent copy streams stream faster than full occupancy (FLUX
+    // cache writes: bf16 sources best at 4 CTAs per SM, fp32 sources at 3)
+    const int cap = sb ? 4 : 3;
+    *smem = (size_t)p->dev.smem_per_sm / (cap + 1);
     int& occ = p->dev.occ_push[sb ? 1 : 0][db ? 1 : 0];
     if (occ == 0) {
-        cudaError_t e = cbk::push_blocks_per_sm(sb, db, &occ);
+        cudaError_t e = cbk::push_blocks_per_sm(sb, db, *smem, &occ);
         if (e != cudaSuccess || occ <= 0) {
             occ = 0;
             return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "occupancy");
         }
     }
-    // fewer concurrent copy streams stream faster than full occupancy (FLUX
-    // cache writes: bf16 sources best at 4 CTAs per SM, fp32 sources at 3)
-    const int cap = sb ? 4 : 3;
-    long long g = (long long)p->dev.sms * (occ < cap ? occ : cap);
+    long long g = (long long)p->dev.sms * occ;
     *grid = (int)(tiles < g ? tiles : g);
     return CB_OK;
 }
@@ -399,6 +402,7 @@ int launch_epilogue(Launch& L, cbk::ExtrapArgs& A) {
     if (r == CB_OK) r = clear_status(L);
     if (r != CB_OK) return r;
     const int grid = (int)std::min<long long>(A.tiles_total, (long long)L.p->dev.sms * occ);
+    A.overlap = 1;
     cudaError_t e = cbk::launch_epilogue(A, grid, (cudaStream_t)L.stream);
     return e == cudaSuccess ? CB_OK : cuda_fail(e, "epilogue launch");
 }
@@ -507,6 +511,10 @@ int launch_bulk(Launch& L, cbk::ExtrapArgs& A, bool strided) {
     // three and fp32 gates lose 1 to 4 % by it).
     if (L.full_step && cb16 && gated && hold && max_nb == 2 && L.gate_dtype == CB_BF16) frac = 0.95;
     const long long ctas = std::max(1LL, (long long)((double)p->dev.sms * per_sm * frac));
+    // An overlapping launch's blocks go wherever they fit: ask for so much shared
+    // memory that no SM takes more than its share of them.
+    A.overlap = frac == 1.0 ? 1 : 0;
+    smem = std::max(smem, (size_t)p->dev.smem_per_sm / (per_sm + 1));
     const int grid = A.any_scalar ? (int)ctas : (int)std::min<long long>((long long)A.tiles_total + A.n_ragged, ctas);
     rc = clear_status(L);
     if (rc != CB_OK) return rc;
@@ -796,14 +804,16 @@ int cb_cache_push(cb_plan* p, const void* const* feats, cb_dtype feat_dtype, dou
     A.tile_begin[n] = (int)tiles;
     A.n_items = n;
     A.tiles_total = (int)tiles;
+    A.overlap = 1;
     int rc = ensure_device(p);
     if (rc != CB_OK) return rc;
     int grid = 0;
-    rc = push_grid(p, sb, db, (int)tiles, &grid);
+    size_t smem = 0;
+    rc = push_grid(p, sb, db, (int)tiles, &grid, &smem);
     if (rc != CB_OK) return rc;
     rc = clear_status_once(p, stream);
     if (rc != CB_OK) return rc;
-    cudaError_t e = cbk::launch_push(A, sb, db, grid, (cudaStream_t)stream);
+    cudaError_t e = cbk::launch_push(A, sb, db, grid, smem, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "push launch");
     // the pair (t, f_t) is now in H; the oldest entry was overwritten when full
     p->slot_t[p->next] = t;

@@ -80,6 +80,7 @@ __device__ __forceinline__ void copy1(unsigned char* dst, const void* src, long 
 template <bool SB, bool DB>
 __global__ void __launch_bounds__(kThreads) push_kernel(const __grid_constant__ PushArgs A) {
     constexpr long long TE = push_tile_elems;
+    after_previous();
     int it = 0;
     for (int tile = blockIdx.x; tile < A.tiles_total; tile += gridDim.x) {
         while (tile >= A.tile_begin[it + 1]) ++it;
@@ -102,26 +103,28 @@ __global__ void __launch_bounds__(kThreads) push_kernel(const __grid_constant__ 
 }
 
 template <bool SB, bool DB>
-cudaError_t launch_t(const PushArgs& a, int grid, cudaStream_t s) {
-    push_kernel<SB, DB><<<grid, kThreads, 0, s>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_t(const PushArgs& a, int grid, size_t smem, cudaStream_t s) {
+    return launch_overlapped(push_kernel<SB, DB>, grid, kThreads, smem, s, a);
 }
 
 template <bool SB, bool DB>
-cudaError_t occ_t(int* blocks) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, push_kernel<SB, DB>, kThreads, 0);
+cudaError_t occ_t(size_t smem, int* blocks) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(push_kernel<SB, DB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, push_kernel<SB, DB>, kThreads, smem);
 }
 
 }  // namespace
 
-cudaError_t launch_push(const PushArgs& a, bool src_bf16, bool dst_bf16, int grid, cudaStream_t s) {
-    if (src_bf16) return dst_bf16 ? launch_t<true, true>(a, grid, s) : launch_t<true, false>(a, grid, s);
-    return dst_bf16 ? launch_t<false, true>(a, grid, s) : launch_t<false, false>(a, grid, s);
+cudaError_t launch_push(const PushArgs& a, bool src_bf16, bool dst_bf16, int grid, size_t smem, cudaStream_t s) {
+    if (src_bf16) return dst_bf16 ? launch_t<true, true>(a, grid, smem, s) : launch_t<true, false>(a, grid, smem, s);
+    return dst_bf16 ? launch_t<false, true>(a, grid, smem, s) : launch_t<false, false>(a, grid, smem, s);
 }
 
-cudaError_t push_blocks_per_sm(bool src_bf16, bool dst_bf16, int* blocks) {
-    if (src_bf16) return dst_bf16 ? occ_t<true, true>(blocks) : occ_t<true, false>(blocks);
-    return dst_bf16 ? occ_t<false, true>(blocks) : occ_t<false, false>(blocks);
+cudaError_t push_blocks_per_sm(bool src_bf16, bool dst_bf16, size_t smem, int* blocks) {
+    if (src_bf16) return dst_bf16 ? occ_t<true, true>(smem, blocks) : occ_t<true, false>(smem, blocks);
+    return dst_bf16 ? occ_t<false, true>(smem, blocks) : occ_t<false, false>(smem, blocks);
 }
 
 }  // namespace cbk

@@ -27,15 +27,23 @@ namespace {
 std::mutex g_mu;
 int* g_addr[cbk::kMaxStatusDevices] = {};
 
-__global__ void take_status_kernel(int* word, int* status) { *status = atomicExch(word, 0); }
+struct Handover {
+    int* word;
+    int* status;
+    int overlap;
+};
+
+__global__ void take_status_kernel(const Handover h) {
+    cbk::after_previous();
+    *h.status = atomicExch(h.word, 0);
+}
 
 }  // namespace
 
 namespace cbk {
 
 cudaError_t take_status(int* word, int* status, cudaStream_t s) {
-    take_status_kernel<<<1, 1, 0, s>>>(word, status);
-    return cudaGetLastError();
+    return launch_overlapped(take_status_kernel, 1, 1, 0, s, Handover{word, status, 1});
 }
 
 cudaError_t noalloc_status_word(int device, int** word) {
