@@ -251,9 +251,12 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
     const int nb = GROUPED ? A.nb[it] : 1;
     const int first = A.first[it];
     void* resid = GROUPED ? A.resid[it] : nullptr;
-    // gates wait in registers through the sums, unless those need the registers
-    // (DiT-XL/2 512^2, K = 8: 785 against 825 us; K = 4: 596 against 589)
-    constexpr bool LATE_GATES = GATED && !RAGGED && K >= 6;
+    // Gates come with the stage (staged_gates), else from global memory, asked
+    // for before the wait, and wait in registers through the sums; with bf16
+    // sources and K >= 6 the sums need those (DiT-XL/2 512^2, K = 8: 785 against
+    // 825 us; K = 4: 596 against 589).
+    constexpr bool LATE_GATES = GATED && !RAGGED && CB16 && K >= 6;
+    constexpr bool STAGED_GATES = GATED && !RAGGED && staged_gates(K, CB16);
     const int held = RAGGED ? (int)ragged_bytes<ES>(A, n) / ES : 0;  // elements in the chunks
     // first element of vector v of this thread, and of pair q of its vector v
     auto at = [&](int v) { return (v * NCT + c) * kVecElems; };
@@ -273,7 +276,7 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
         long long ev[U];
 #pragma unroll
         for (int v = 0; v < U; ++v) ev[v] = e0 + at(v);
-        if (gated) gate_offsets<U>(A, it, e0, ev, gi);
+        if (gated) gate_offsets<U>(A, it, e0, ev, gi, STAGED_GATES && A.stage_gate_bytes != 0);
     }
     // ragged: of the pairs' first elements, and whether the second one lies in
     // the next token of the same batch, hidden channels back
@@ -299,13 +302,12 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
         });
 #pragma unroll 1
     for (int m = 0; m < nb; ++m) {
-        // gates from global memory, asked for before the wait for the stage
         float g[U][8];
         if constexpr (GATED) {
             const void* gp = gated ? A.m_gate[first + m] : nullptr;
 #pragma unroll
             for (int v = 0; v < U; ++v) {
-                if (LATE_GATES) continue;
+                if (LATE_GATES || STAGED_GATES) continue;
                 if (!RAGGED && gp != nullptr) {
                     load_x8(gp, A.gate_bf16, (long long)gi[v], g[v]);
                     continue;
@@ -352,6 +354,18 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
                     }
                 }
             }
+        if constexpr (STAGED_GATES) {  // rows that came with the stage, or from global memory
+            const void* gp = gated ? A.m_gate[first + m] : nullptr;
+            if (gp != nullptr && A.stage_gate_bytes) gp = base + K * Sh::chunk + A.stage_x_bytes;
+#pragma unroll
+            for (int v = 0; v < U; ++v) {
+                if (gp != nullptr)
+                    load_x8(gp, A.gate_bf16, (long long)gi[v], g[v]);
+                else
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) g[v][e] = 1.0f;
+            }
+        }
         if (GROUPED && !RAGGED && m == 0 && resid != nullptr)
             resid_begin<U>(acc, [&](int v, float (&x)[8]) {
                 if (A.stage_x_bytes)

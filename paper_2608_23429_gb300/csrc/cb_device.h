@@ -154,9 +154,17 @@ struct BulkShape {
     int consumer_warps;
     int tile;
 };
+// Compensated launches whose gate rows are staged with their member: where the
+// loads' latency counts more than the rows' room and traffic (GB300, 28 groups of
+// two, [8, 256, 1152]: fp32 sources, K = 1 and 2 343 -> 268 and 380 -> 313 us,
+// K = 4 481 -> 460 us; bf16 sources and gates, K = 1 and 2 240 -> 226 and 305 ->
+// 289 us, but with fp32 gates 280 -> 287 us for K = 2 and 586 -> 633 us for K = 4,
+// [4, 1024, 1152]).
+__host__ __device__ constexpr bool staged_gates(int K, bool src_bf16) { return !src_bf16 || K <= 2; }
 __host__ __device__ constexpr BulkShape bulk_shape(int K, bool src_bf16, bool grouped, bool gated, bool precise) {
+    // fp32 sources with gates and K <= 2: 15 warps (K = 1: 374 -> 343 us)
     if (precise) {
-        const int warps = src_bf16 ? 19 : 11;
+        const int warps = src_bf16 ? 19 : gated && K <= 2 ? 15 : 11;
         return BulkShape{1, warps, warps * 32 * kVecElems};
     }
     const bool two = (K == 1 && !(src_bf16 && grouped && !gated)) || (src_bf16 && !grouped && K <= 2) ||

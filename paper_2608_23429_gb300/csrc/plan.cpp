@@ -432,9 +432,9 @@ int launch_bulk(Launch& L, cbk::ExtrapArgs& A, bool strided) {
     A.stage_gate_bytes = 0;
     const bool hold = grouped && !precise;
     const int min_stages = hold ? max_nb + 1 : 2;
-    // gate rows travel with their member when every gated tile touches at
-    // most two batches (a batch holds a tile or more) and two rows are small
-    if (gated && !precise) {
+    // Gate rows travel with their member when every gated tile touches at
+    // most two batches (a batch holds a tile or more) and two rows are small.
+    if (gated && !strided && (!precise || cbk::staged_gates(K, cb16))) {
         const size_t gs = esize(L.gate_dtype);
         size_t need = 0;
         bool fits = true;
