@@ -58,9 +58,9 @@ namespace {
 // consumer warps per SM (two independent pipelines), bf16 threads taking two
 // vectors per tile. An earlier map of 8 consumer warps with two vectors each
 // on one CTA left the launches with hidden states issue-bound.
-template <bool CB16, int K, bool GROUPED, bool GATED, bool PRECISE>
+template <bool CB16, int K, bool GROUPED, bool GATED, bool PRECISE, bool STRIDED = false>
 struct Shape {
-    static constexpr BulkShape b = bulk_shape(K, CB16, GROUPED, GATED, PRECISE);
+    static constexpr BulkShape b = bulk_shape(K, CB16, GROUPED, GATED, PRECISE, STRIDED);
     static constexpr int ctas_per_sm = b.ctas_per_sm;
     static constexpr int consumer_warps = b.consumer_warps;
     static constexpr int consumers = consumer_warps * 32;
@@ -98,10 +98,9 @@ __device__ __forceinline__ uint32_t ragged_bytes(const ExtrapArgs& A, long long 
 
 // The producer lane: every unit's history chunks, and what travels with them,
 // from global into shared memory, in the consumers' order.
-template <int K, bool CB16, bool GROUPED, bool GATED, bool PRECISE, bool STRIDED>
+template <typename Sh, int K, bool CB16, bool GROUPED, bool GATED>
 __device__ __forceinline__ void produce(const ExtrapArgs& A, uint32_t full0, uint32_t empty0, uint32_t buf0,
                                         uint32_t stage_bytes) {
-    using Sh = Shape<CB16, K, GROUPED, GATED, PRECISE>;
     constexpr long long TE = Sh::tile;
     constexpr int ES = CB16 ? 2 : 4;
     const int S = A.stages;
@@ -159,9 +158,7 @@ __device__ __forceinline__ void produce(const ExtrapArgs& A, uint32_t full0, uin
     bool ok = true;
     for (; ok && tile < A.tiles_total; tile += gridDim.x) {
         while (tile >= A.tile_begin[it + 1]) ++it;
-        const long long e0 = (long long)(tile - A.tile_begin[it]) * TE;
-        const bool whole = !STRIDED || e0 + TE <= A.numel[it];
-        ok = issue(it, e0, whole, whole ? (uint32_t)Sh::chunk : ragged_bytes<ES>(A, A.numel[it] - e0));
+        ok = issue(it, (long long)(tile - A.tile_begin[it]) * TE, true, (uint32_t)Sh::chunk);
     }
 #pragma unroll 1
     for (; ok && tile < A.tiles_total + A.n_ragged; tile += gridDim.x) {
@@ -205,21 +202,19 @@ __device__ __forceinline__ uint2 ragged_pair(const unsigned char* p, int i, int 
     return w;
 }
 
-// Four pairs of elements p[at(q, 0)], p[at(q, 1)]; 0 where at() is negative.
-template <typename At>
-__device__ __forceinline__ void read_pairs(const void* p, bool bf16, float (&x)[8], At at) {
+// Four pairs of elements p[at(q, 0)], p[at(q, 1)]; 0 where in(q, e) is false.
+template <typename At, typename In>
+__device__ __forceinline__ void read_pairs(const void* p, bool bf16, float (&x)[8], At at, In in) {
     if (bf16) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const long long e = at(i >> 1, i & 1);
-            x[i] = e >= 0 ? __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(p)[e] << 16) : 0.0f;
-        }
+        for (int i = 0; i < 8; ++i)
+            x[i] = in(i >> 1, i & 1)
+                       ? __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(p)[at(i >> 1, i & 1)] << 16)
+                       : 0.0f;
     } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const long long e = at(i >> 1, i & 1);
-            x[i] = e >= 0 ? reinterpret_cast<const float*>(p)[e] : 0.0f;
-        }
+        for (int i = 0; i < 8; ++i)
+            x[i] = in(i >> 1, i & 1) ? reinterpret_cast<const float*>(p)[at(i >> 1, i & 1)] : 0.0f;
     }
 }
 
@@ -235,12 +230,12 @@ __device__ __forceinline__ void read_pairs(const void* p, bool bf16, float (&x)[
 // adjacent threads on adjacent pairs, so that any length is covered from
 // shared memory with the same arithmetic (and bits).
 //
-// precise_tile: one tile of one item. RAGGED: any length n <= tile, pairs as
-// above. False when a wait ran out.
+// precise_tile: one tile of one item. RAGGED: pairs as above; FULL: of a whole
+// tile, else of any length n. False when a wait ran out.
 struct Cursor {
     uint32_t stage = 0, phase = 0;  // of the next unit to consume
 };
-template <typename Sh, int K, bool CB16, bool GROUPED, bool GATED, bool RAGGED>
+template <typename Sh, int K, bool CB16, bool GROUPED, bool GATED, bool RAGGED, bool FULL = !RAGGED>
 __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long long e0, int n, Cursor& cur,
                                              uint32_t full0, uint32_t empty0, const unsigned char* stages,
                                              uint32_t stage_bytes, int lane) {
@@ -257,7 +252,8 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
     // 825 us; K = 4: 596 against 589).
     constexpr bool LATE_GATES = GATED && !RAGGED && CB16 && K >= 6;
     constexpr bool STAGED_GATES = GATED && !RAGGED && staged_gates(K, CB16);
-    const int held = RAGGED ? (int)ragged_bytes<ES>(A, n) / ES : 0;  // elements in the chunks
+    const int held = RAGGED && !FULL ? (int)ragged_bytes<ES>(A, n) / ES : Sh::tile;  // elements in the chunks
+    auto in = [&](int i) { return FULL || i < n; };
     // first element of vector v of this thread, and of pair q of its vector v
     auto at = [&](int v) { return (v * NCT + c) * kVecElems; };
     auto pair_at = [&](int v, int q) { return 2 * (c + NCT * (4 * v + q)); };
@@ -265,9 +261,10 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
         if constexpr (!RAGGED) {
             store_o8(p, bf16, e0 + at(v), o);
         } else {
+            unsigned char* base = reinterpret_cast<unsigned char*>(p) + e0 * (bf16 ? 2 : 4);
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                store_o2(p, bf16, e0 + pair_at(v, q), n - pair_at(v, q), bf16 ? o[q] : o[2 * q], o[2 * q + 1]);
+                store_o2(base, bf16, pair_at(v, q), FULL ? 2 : n - pair_at(v, q), bf16 ? o[q] : o[2 * q], o[2 * q + 1]);
         }
     };
     const bool gated = GATED && resid != nullptr && A.i_row[it] != 0;  // items without a shape carry no gate
@@ -280,6 +277,7 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
     }
     // ragged: of the pairs' first elements, and whether the second one lies in
     // the next token of the same batch, hidden channels back
+    const unsigned hidden = GATED && RAGGED ? A.i_hidden[it] : 0u;
     unsigned gq[U][4], back = 0u;
     if constexpr (GATED && RAGGED) {
         if (gated)
@@ -288,7 +286,7 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     bool b;
-                    gate_offset_pair(A, it, e0 + (pair_at(v, q) < n ? pair_at(v, q) : 0), gq[v][q], b);
+                    gate_offset_pair(A, it, e0 + (in(pair_at(v, q)) ? pair_at(v, q) : 0), gq[v][q], b);
                     back |= b ? 1u << (4 * v + q) : 0u;
                 }
     }
@@ -296,9 +294,9 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
     Finite fin;
     if (GROUPED && RAGGED && resid != nullptr)  // not staged: asked for before the wait for the stage
         resid_begin<U>(acc, [&](int v, float (&x)[8]) {
-            read_pairs(resid, A.resid_bf16, x, [&](int q, int e) {
-                return pair_at(v, q) + e < n ? e0 + pair_at(v, q) + e : -1ll;
-            });
+            read_pairs(
+                reinterpret_cast<const unsigned char*>(resid) + e0 * (A.resid_bf16 ? 2 : 4), A.resid_bf16, x,
+                [&](int q, int e) { return pair_at(v, q) + e; }, [&](int q, int e) { return in(pair_at(v, q) + e); });
         });
 #pragma unroll 1
     for (int m = 0; m < nb; ++m) {
@@ -315,10 +313,10 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
 #pragma unroll
                 for (int e = 0; e < 8; ++e) g[v][e] = 1.0f;
                 if (RAGGED && gp != nullptr)
-                    read_pairs(gp, A.gate_bf16, g[v], [&](int q, int e) {
-                        const long long at = gq[v][q] + e - (e && (back >> (4 * v + q) & 1u) ? A.i_hidden[it] : 0u);
-                        return pair_at(v, q) + e < n ? at : -1ll;
-                    });
+                    read_pairs(
+                        gp, A.gate_bf16, g[v],
+                        [&](int q, int e) { return gq[v][q] + e - (e && (back >> (4 * v + q) & 1u) ? hidden : 0u); },
+                        [&](int q, int e) { return in(pair_at(v, q) + e); });
             }
         }
         const uint32_t stage = cur.stage;
@@ -345,7 +343,7 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
                     const unsigned char* src = hist_ptr(A, j, A.m_off[first + m]) + e0 * ES;
                     uint2 w[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) w[q] = ragged_pair<CB16, K == 1>(chunk, pair_at(v, q), n, held, src);
+                    for (int q = 0; q < 4; ++q) w[q] = ragged_pair<CB16, K == 1 && !FULL>(chunk, pair_at(v, q), FULL ? Sh::tile : n, held, src);
                     if constexpr (CB16) {
                         raw[v][j][0] = make_uint4(w[0].x, w[1].x, w[2].x, w[3].x);
                     } else {
@@ -409,7 +407,7 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
 #pragma unroll 1
             for (int e = 0; e < kVecElems; ++e) {
                 const int i = RAGGED ? pair_at(v, e >> 1) + (e & 1) : at(v) + e;
-                if (i < n) scalar_element<CB16>(A, K, it, e0 + i);
+                if (in(i)) scalar_element<CB16>(A, K, it, e0 + i);
             }
     }
     return true;
@@ -605,13 +603,13 @@ __device__ __forceinline__ bool fast_tiles(const ExtrapArgs& A, int& tile, Curso
 // hold no whole vectors), every tile by pairs of elements. Compiled apart so
 // that each kernel carries only its own path.
 template <int K, bool CB16, bool GROUPED, bool GATED, bool ONE = false, bool PRECISE = false, bool STRIDED = false>
-__global__ void __launch_bounds__(Shape<CB16, K, GROUPED, GATED, PRECISE>::threads,
-                                  Shape<CB16, K, GROUPED, GATED, PRECISE>::ctas_per_sm)
+__global__ void __launch_bounds__(Shape<CB16, K, GROUPED, GATED, PRECISE, STRIDED>::threads,
+                                  Shape<CB16, K, GROUPED, GATED, PRECISE, STRIDED>::ctas_per_sm)
     extrapolate_bulk_kernel(const __grid_constant__ ExtrapArgs A) {
     static_assert(!ONE || (K == 1 && !PRECISE), "the epilogue is a one-entry history");
     static_assert(!STRIDED || PRECISE, "strided tiles are compensated");
     extern __shared__ __align__(128) unsigned char smem[];
-    using Sh = Shape<CB16, K, GROUPED, GATED, PRECISE>;
+    using Sh = Shape<CB16, K, GROUPED, GATED, PRECISE, STRIDED>;
     constexpr int NCW = Sh::consumer_warps;
     constexpr long long TE = Sh::tile;
     const int S = A.stages;
@@ -635,7 +633,7 @@ __global__ void __launch_bounds__(Shape<CB16, K, GROUPED, GATED, PRECISE>::threa
         (uint32_t)K * Sh::chunk + (!GROUPED ? 0u : PRECISE ? A.stage_x_bytes : (uint32_t)Sh::tile * 2u);
     const uint32_t stage_bytes = gates_at + (GATED ? A.stage_gate_bytes : 0u);
     if (warp == NCW) {
-        if (lane == 0) produce<K, CB16, GROUPED, GATED, PRECISE, STRIDED>(A, full0, empty0, buf0, stage_bytes);
+        if (lane == 0) produce<Sh, K, CB16, GROUPED, GATED>(A, full0, empty0, buf0, stage_bytes);
         return;
     }
     const unsigned char* stages = smem + kBarrierBytes;
@@ -646,18 +644,16 @@ __global__ void __launch_bounds__(Shape<CB16, K, GROUPED, GATED, PRECISE>::threa
         for (; tile < A.tiles_total; tile += gridDim.x) {
             while (tile >= A.tile_begin[it + 1]) ++it;
             const long long e0 = (long long)(tile - A.tile_begin[it]) * TE;
-            const int n = STRIDED && A.numel[it] - e0 < TE ? (int)(A.numel[it] - e0) : (int)TE;
-            if (!precise_tile<Sh, K, CB16, GROUPED, GATED, STRIDED>(A, it, e0, n, cur, full0, empty0, stages,
-                                                                    stage_bytes, lane))
+            if (!precise_tile<Sh, K, CB16, GROUPED, GATED, STRIDED, true>(A, it, e0, (int)TE, cur, full0, empty0, stages,
+                                                                          stage_bytes, lane))
                 return;
         }
-        if constexpr (STRIDED) return;
     } else if (!fast_tiles<K, CB16, GROUPED, GATED, ONE>(A, tile, cur, full0, empty0, stages, stage_bytes, gates_at,
                                                          lane)) {
         return;
     }
     if (!ragged_tiles<Sh, K, CB16, GROUPED, GATED>(A, tile, cur, full0, empty0, stages, stage_bytes, lane)) return;
-    scalar_items<Sh, K, CB16>(A);
+    if constexpr (!STRIDED) scalar_items<Sh, K, CB16>(A);
 }
 
 }  // namespace

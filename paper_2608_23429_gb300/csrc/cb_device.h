@@ -161,10 +161,13 @@ struct BulkShape {
 // 289 us, but with fp32 gates 280 -> 287 us for K = 2 and 586 -> 633 us for K = 4,
 // [4, 1024, 1152]).
 __host__ __device__ constexpr bool staged_gates(int K, bool src_bf16) { return !src_bf16 || K <= 2; }
-__host__ __device__ constexpr BulkShape bulk_shape(int K, bool src_bf16, bool grouped, bool gated, bool precise) {
-    // fp32 sources with gates and K <= 2: 15 warps (K = 1: 374 -> 343 us)
+__host__ __device__ constexpr BulkShape bulk_shape(int K, bool src_bf16, bool grouped, bool gated, bool precise,
+                                                   bool strided) {
+    // fp32 sources with gates and K <= 2: 15 warps (K = 1: 374 -> 343 us); so for
+    // the strided kernels with hidden states, which hold more (8 x 3 x [3, 333,
+    // 577], gates: 63.7 -> 59.8 us, K = 8 75 -> 70 us, [8, 333, 577] the same)
     if (precise) {
-        const int warps = src_bf16 ? 19 : gated && K <= 2 ? 15 : 11;
+        const int warps = src_bf16 ? (strided && grouped ? 15 : 19) : gated && K <= 2 ? 15 : 11;
         return BulkShape{1, warps, warps * 32 * kVecElems};
     }
     const bool two = (K == 1 && !(src_bf16 && grouped && !gated)) || (src_bf16 && !grouped && K <= 2) ||

@@ -12,7 +12,7 @@ namespace {
 template <int K, bool CB16, bool GROUPED, bool GATED, bool STRIDED>
 cudaError_t launch_one(const ExtrapArgs& a, int grid, size_t smem, cudaStream_t s) {
     return launch_overlapped(extrapolate_bulk_kernel<K, CB16, GROUPED, GATED, false, true, STRIDED>, grid,
-                             Shape<CB16, K, GROUPED, GATED, true>::threads, smem, s, a);
+                             Shape<CB16, K, GROUPED, GATED, true, STRIDED>::threads, smem, s, a);
 }
 
 template <int K, bool CB16, bool STRIDED>

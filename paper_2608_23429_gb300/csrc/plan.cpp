@@ -325,13 +325,13 @@ int clear_status(Launch& L) {
 
 // Cut the items into tiles of te elements, numbered across items. `split` (the
 // bulk kernel's numbering): whole tiles first, then the ragged last ones;
-// items off the 16-byte grid have none.
-int cut_tiles(cbk::ExtrapArgs& A, long long te, bool split) {
+// items with vec_ok = 0 have none, unless the launch is `strided`.
+int cut_tiles(cbk::ExtrapArgs& A, long long te, bool split, bool strided = false) {
     long long tiles = 0;
     A.n_ragged = A.any_scalar = 0;
     for (int i = 0; i < A.n_items; ++i) {
         A.tile_begin[i] = (int)tiles;
-        if (split && !A.vec_ok[i]) {
+        if (split && !strided && !A.vec_ok[i]) {
             A.any_scalar = 1;
             continue;
         }
@@ -421,8 +421,8 @@ int launch_bulk(Launch& L, cbk::ExtrapArgs& A, bool strided) {
         any_resid = any_resid || A.resid[i] != nullptr;
         grouped = grouped || A.resid[i] != nullptr || A.nb[i] > 1;
     }
-    const cbk::BulkShape shape = cbk::bulk_shape(K, cb16, grouped, gated, precise);
-    int rc = cut_tiles(A, shape.tile, !strided);
+    const cbk::BulkShape shape = cbk::bulk_shape(K, cb16, grouped, gated, precise, strided);
+    int rc = cut_tiles(A, shape.tile, true, strided);
     if (rc != CB_OK) return rc;
     // Hidden states travel through shared memory with the first member of their
     // group (not those off the 16-byte grid). Launches that recompute guarded
