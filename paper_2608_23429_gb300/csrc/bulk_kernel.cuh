@@ -107,7 +107,8 @@ __device__ __forceinline__ void produce(const ExtrapArgs& A, uint32_t full0, uin
     unsigned u = 0;               // units issued
     uint32_t ps = 0, wraps = 0;   // stage of the next unit; times the ring has wrapped
     // one tile of item `it`: a unit per member; false when a wait ran out
-    auto issue = [&](int it, long long e0, bool whole, uint32_t bytes) {
+    const uint64_t normal = policy_normal(), passing = policy_first();
+    auto issue = [&](int it, long long e0, bool whole, uint32_t bytes, uint64_t policy) {
         const int first = A.first[it];
         const int nb = GROUPED ? A.nb[it] : 1;
         const unsigned char* resid = GROUPED ? reinterpret_cast<const unsigned char*>(A.resid[it]) : nullptr;
@@ -143,14 +144,15 @@ __device__ __forceinline__ void produce(const ExtrapArgs& A, uint32_t full0, uin
 #pragma unroll
                 for (int j = 0; j < K; ++j)
                     bulk_g2s(dst + j * (uint32_t)Sh::chunk, hist_ptr(A, j, A.m_off[first + m]) + e0 * ES, bytes,
-                             full0 + 8u * stage);
+                             full0 + 8u * stage, policy);
             }
             if (xbytes)
                 bulk_g2s(dst + K * (uint32_t)Sh::chunk, resid + e0 * (A.resid_bf16 ? 2 : 4), xbytes,
-                         full0 + 8u * stage);
+                         full0 + 8u * stage, normal);
             if (gb)
                 bulk_g2s(dst + K * (uint32_t)Sh::chunk + A.stage_x_bytes,
-                         reinterpret_cast<const unsigned char*>(A.m_gate[first + m]) + gsrc, gb, full0 + 8u * stage);
+                         reinterpret_cast<const unsigned char*>(A.m_gate[first + m]) + gsrc, gb, full0 + 8u * stage,
+                         normal);
         }
         return true;
     };
@@ -158,13 +160,14 @@ __device__ __forceinline__ void produce(const ExtrapArgs& A, uint32_t full0, uin
     bool ok = true;
     for (; ok && tile < A.tiles_total; tile += gridDim.x) {
         while (tile >= A.tile_begin[it + 1]) ++it;
-        ok = issue(it, (long long)(tile - A.tile_begin[it]) * TE, true, (uint32_t)Sh::chunk);
+        ok = issue(it, (long long)(tile - A.tile_begin[it]) * TE, true, (uint32_t)Sh::chunk,
+                   tile < A.keep_tiles ? normal : passing);
     }
 #pragma unroll 1
     for (; ok && tile < A.tiles_total + A.n_ragged; tile += gridDim.x) {
         it = A.ragged[tile - A.tiles_total];
         const long long e0 = (long long)(A.tile_begin[it + 1] - A.tile_begin[it]) * TE;
-        ok = issue(it, e0, false, ragged_bytes<ES>(A, A.numel[it] - e0));
+        ok = issue(it, e0, false, ragged_bytes<ES>(A, A.numel[it] - e0), normal);
     }
     // never leave while copies into this CTA's shared memory are in flight:
     // wait for every unit still in the ring; after one wait runs out (a unit

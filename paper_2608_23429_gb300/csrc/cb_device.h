@@ -81,6 +81,7 @@ struct ExtrapArgs {
     int* status;                 // bulk variant: device status word (codes OR-ed in)
     int overlap;                 // host only: see launch_overlapped
     int withhold_first;          // bulk variant, tests only: announce but never issue the first copies
+    int keep_tiles;              // bulk variant: whole tiles whose history L2 is to keep for the next step
     // bulk variant: tile_begin and tiles_total count whole tiles only (none of
     // items with vec_ok = 0); the ragged last tiles are numbered after them
     int n_ragged;
