@@ -150,3 +150,33 @@ def test_full_step_beside_off_grid_hidden_states(cb, H, src, io):
             assert st["bad"] == 0, (k, g, st)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("steps", [1, 12])
+def test_steps_in_a_row_match_the_direct_kernel(cb, H, steps):
+    """Launches that overlap the end of the one before, each adding to the
+    hidden states that it left, with a history a little larger than L2's share
+    for it (71 MB, most of it copied in for eviction first): bit for bit what
+    the direct-load kernel gives, which overlaps nothing."""
+    tensors = [workloads.TensorSpec(g, b, (1, 256, 1152), g) for g in range(15) for b in range(2)]
+    w = workloads.Workload(name="row", tensors=tensors, K=4, cache_dtype="bf16", T=0, r=0, t_min=0.0, t_max=999.0,
+                           timesteps=[], degree=6, noise=0.1, seed=41)
+    nodes = [900.0, 860.0, 820.0, 780.0]
+    got = {}
+    for kernel in ("auto", "direct"):
+        walk = H.Walk(w, node_t=nodes, kernel=kernel)
+        feats = [[workloads.trajectory(w, i, t, k, "cuda") for i in range(len(tensors))] for k, t in enumerate(nodes)]
+        resid = [workloads.hidden_state(w, g, "cuda") for g in range(walk.n_groups)]
+        outs = [torch.empty(s.shape, dtype=torch.bfloat16, device="cuda") for s in tensors]
+        for t, f in zip(nodes, feats):
+            cb.cb_cache_push(walk.plan, f, cb.CB_BF16, t)
+        for k in range(steps):
+            cb.cb_extrapolate(walk.plan, 770.0 - k, outs, cb.CB_BF16, resid, cb.CB_BF16)
+        cb.cb_cache_push(walk.plan, outs, cb.CB_BF16, 700.0)  # the last predictions, as a full step's features
+        torch.cuda.synchronize()
+        assert cb.cb_plan_device_status(walk.plan) == 0
+        got[kernel] = (outs, resid, walk.cache[: walk.cache.numel() - cb.CB_STATUS_BYTES])
+        walk.close()
+    for a, b in zip(got["auto"][0] + got["auto"][1], got["direct"][0] + got["direct"][1]):
+        assert torch.equal(a.view(torch.int16), b.view(torch.int16))
+    assert torch.equal(got["auto"][2], got["direct"][2])
