@@ -63,7 +63,7 @@ NOMINAL_HBM_GBS = 7900.0
 KERNEL_SOURCES = ["paper_2608_23429_gb300/csrc/extrapolate_bulk.cu", "paper_2608_23429_gb300/csrc/bulk_kernel.cuh",
                   "paper_2608_23429_gb300/csrc/extrapolate.cu", "paper_2608_23429_gb300/csrc/direct_kernel.cuh",
                   "paper_2608_23429_gb300/csrc/cb_math.cuh", "paper_2608_23429_gb300/csrc/cb_device.h",
-                  "paper_2608_23429_gb300/csrc/cb_async.cuh"]
+                  "paper_2608_23429_gb300/csrc/cb_async.cuh", "paper_2608_23429_gb300/csrc/extrapolate_bulk_precise.cuh"]
 
 
 def kernel_hash() -> str:

@@ -36,7 +36,7 @@
  *   - Layout: each branch tensor is a contiguous row-major array
  *     [batch, tokens, hidden] of `numel` elements. Pointers must be aligned to
  *     their element size; pointers aligned to 16 bytes take the vectorised
- *     path, others a scalar path (same results).
+ *     path, others paths by elements or pairs of them (same accuracy).
  *   - Rounding: fp32 -> bf16 conversions round to nearest, ties to even.
  */
 #ifndef CHEBBOOST_H

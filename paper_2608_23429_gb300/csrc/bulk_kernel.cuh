@@ -3,15 +3,19 @@
 // compensated path for every element here. Sec. 3.3, Eq. for f_t; Alg. 1,
 // extrapolation branch).
 //
-// One or two CTAs per SM (see Shape). A producer lane moves,
-// for every work unit (one tile of one branch tensor), the K history chunks of
-// 8 KB each from HBM into a ring of shared-memory stages with cp.async.bulk
-// (the Blackwell bulk-copy engine), each stage guarded by a "full" mbarrier
-// (transaction bytes) and an "empty" mbarrier (one arrival per consumer warp).
-// Consumer warps read their 8-element vectors of the K chunks from shared
-// memory, compute, and store from registers. With S stages of K x 8 KB (S = 5
-// for K = 5) up to ~200 KB per SM stay in flight independently of the
-// consumers' registers, which is what bounds the direct-load variant.
+// One or two CTAs per SM (see Shape). A producer lane moves, for every work unit
+// (one tile of one branch tensor), the K history chunks of the tile (8 KB each,
+// less or more in the compensated kernels) from HBM into a ring of shared-memory
+// stages with cp.async.bulk (the Blackwell bulk-copy engine), each stage guarded
+// by a "full" mbarrier (transaction bytes) and an "empty" mbarrier (one arrival
+// per consumer warp). Consumer warps read their 8-element vectors of the K
+// chunks from shared memory, compute, and store from registers, so that what is
+// in flight does not depend on the consumers' registers, which bound the
+// direct-load variant. How much is in flight the host decides (launch_bulk).
+//
+// Whole tiles come first, in a loop that tests no lengths; the ragged last tiles
+// follow in a loop of their own (ragged_tiles), and items whose sources are off
+// the 16-byte grid last, without the pipeline (scalar_items).
 //
 // Many consumer warps per scheduler hide the consumers' fixed latencies (see
 // Shape for the thread map). Every consumer fences its reads of a stage
@@ -28,8 +32,9 @@
 //     producer). With gates, each member's stage also carries the gate rows
 //     of the batches its tile touches, so that no consumer waits on a global
 //     load.
-// Launches with fp32 predictions or hidden states (PRECISE) have kernels of
-// their own: see precise_tile.
+// Launches with fp32 predictions or hidden states (PRECISE) and items off the
+// 16-byte grid on their way out (STRIDED) have kernels of their own: see
+// precise_tile.
 // The same kernel runs a full step's epilogue (cb_cache_push_residual) as a
 // one-entry history of weight 1 whose member addresses are the new features;
 // with copy_out the outputs (the ring slot) receive the features converted.
@@ -224,9 +229,11 @@ __device__ __forceinline__ void read_pairs(const void* p, bool bf16, float (&x)[
 // The consumers of launches with fp32 predictions or hidden states: every
 // element takes the compensated sum (sum_vec), so nothing is recomputed and
 // each stage goes back to the producer as soon as its values, and the hidden
-// state behind the first member's, are in registers. The arithmetic (five
-// packed or scalar FMA-pipe operations per history value and element) bounds
-// these launches, not HBM alone.
+// state behind the first member's, are in registers. Predictions alone stream
+// at the copy rate (DiT-XL/2 512^2, K = 8, bf16 history, fp32 predictions: 1180 us
+// with Dot2 in the common kernel, 740 us here, 7.1 TB/s); with gated fp32 hidden
+// states the consumers' latency bounds them (K = 4: 897 -> 584 us, 5.4 TB/s at 57 %
+// of the issue slots).
 //
 // A thread holds vecs vectors of eight elements. In a whole tile they are
 // contiguous; in the ragged last tile of a tensor they are four pairs each,

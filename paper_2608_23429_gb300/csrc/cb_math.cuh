@@ -601,8 +601,9 @@ __device__ __forceinline__ void resid_fast(const ExtrapArgs& A, int it, const lo
 // SIAM J. Sci. Comput. 31(1), 2008, with the product folded into the FMA).
 // Five operations per term against Dot2's eleven: with fp32 results the
 // kernels are bound by the FMA pipe. s + c is within 2^-40 sum_j |w_j F_j| of
-// the exact value (Dot2: 2^-45; 2^6 million sums, K = 3..8, bf16 and fp32
-// features), and the fp32 results' 2-norm error equals Dot2's to seven digits.
+// the exact value (Dot2: 2^-45; 7e7 sums against quad precision, K = 3..8, bf16
+// and fp32 features), and the fp32 results' 2-norm error equals Dot2's to seven
+// digits.
 // Where M overflows (W max |F| >= 2^126) or a feature is not finite, s is not
 // finite: the callers then take scalar_element, which has no anchor.
 //
