@@ -232,7 +232,7 @@ __device__ __forceinline__ void read_pairs(const void* p, bool bf16, float (&x)[
 // state behind the first member's, are in registers. Predictions alone stream
 // at the copy rate (DiT-XL/2 512^2, K = 8, bf16 history, fp32 predictions: 1180 us
 // with Dot2 in the common kernel, 740 us here, 7.1 TB/s); with gated fp32 hidden
-// states the consumers' latency bounds them (K = 4: 897 -> 584 us, 5.4 TB/s at 57 %
+// states the consumers' latency bounds them (K = 4: 897 -> 528 us, 6.0 TB/s at 57 %
 // of the issue slots).
 //
 // A thread holds vecs vectors of eight elements. In a whole tile they are
@@ -258,9 +258,9 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
     void* resid = GROUPED ? A.resid[it] : nullptr;
     // Gates come with the stage (staged_gates), else from global memory, asked
     // for before the wait, and wait in registers through the sums; with bf16
-    // sources and K >= 6 the sums need those (DiT-XL/2 512^2, K = 8: 785 against
-    // 825 us; K = 4: 596 against 589).
-    constexpr bool LATE_GATES = GATED && !RAGGED && CB16 && K >= 6;
+    // sources and K >= 7 the sums need those (DiT-XL/2 512^2, K = 8: 763 against
+    // 779 us; K = 6: 671 against 645, K = 4: 536 against 528).
+    constexpr bool LATE_GATES = GATED && !RAGGED && CB16 && K >= 7;
     constexpr bool STAGED_GATES = GATED && !RAGGED && staged_gates(K, CB16);
     const int held = RAGGED && !FULL ? (int)ragged_bytes<ES>(A, n) / ES : Sh::tile;  // elements in the chunks
     auto in = [&](int i) { return FULL || i < n; };
@@ -395,7 +395,7 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
                 want = false;
             }
         }
-        member_precise<K, CB16, U, GATED>(
+        member_precise<K, CB16, U, GATED, GROUPED>(
             A, want, raw, resid != nullptr, acc, fin,
             [&](int v, float (&gv)[8]) {
                 if constexpr (GATED) {
@@ -407,10 +407,10 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
                         for (int e = 0; e < 8; ++e) gv[e] = LATE_GATES ? 1.0f : g[v][e];
                 }
             },
-            [&](int v, const uint32_t (&o)[8]) { put(out, A.out_bf16, v, o); });
+            [&](int v, bool bf16, const uint32_t (&o)[8]) { put(out, bf16, v, o); });
     }
     if (resid != nullptr ? !resid_precise<K, U>(A, acc, fin,
-                                                [&](int v, const uint32_t (&o)[8]) { put(resid, A.resid_bf16, v, o); })
+                                                [&](int v, bool bf16, const uint32_t (&o)[8]) { put(resid, bf16, v, o); })
                          : !fin.all()) {
 #pragma unroll 1
         for (int v = 0; v < U; ++v)

@@ -689,35 +689,60 @@ struct Finite {
 };
 
 // Compensated path for one member (any launch with fp32 predictions or hidden
-// states): the prediction's output elements to put(u, o) when wanted (o as
+// states): the prediction's output elements to put(u, bf16, o) when wanted (o as
 // put_pair leaves it, for vector u), and accumulation into acc.
-template <int K, bool CB16, int UV, bool GATED, typename Gate, typename Put>
+//
+// The output type and what is wanted are asked once per vector, not per pair:
+// branches between the pairs kept their chains from overlapping and held 10 to
+// 30 registers more (gated fp32 hidden states, DiT-XL/2 512^2: K = 2 520 -> 430 us,
+// K = 4 585 -> 528, K = 8 798 -> 765; the off-grid gated step of 24 x [3, 333, 577]
+// 54 -> 48; a full step of DiT-XL/2 256^2 with fp32 hidden states and gates 230 -> 198).
+// Predictions alone (!GROUPED) with K = 5, 6 and 8, which HBM bounds, stream
+// better with a branch per pair, which spreads the consumers' stores (K = 8
+// 738 against 752 us, K = 6 585 against 608, K = 5 564 against 573; K = 7 704 against 670
+// and K = 4 504 against 496 the other way).
+template <int K, bool CB16, int UV, bool GATED, bool GROUPED, typename Gate, typename Put>
 __device__ __forceinline__ void member_precise(const ExtrapArgs& A, bool want, const RawVecs<K, CB16, UV>& raw,
                                                bool accumulate, Acc<UV>& acc, Finite& fin, Gate gate, Put put) {
 #pragma unroll
     for (int u = 0; u < UV; ++u) {
-        uint32_t o[8];
         float2 sv[4], cv[4];
         sum_vec<K, CB16>(A, raw[u], sv, cv);
         float g[8];
         if constexpr (GATED)
             if (accumulate) gate(u, g);
+        if (want) {
+            uint32_t o[8];
+            auto pair = [&](bool bf16, int q) {
+                float2 hi = add2(sv[q], cv[q]), lo = hi;
+                if (bf16) two_sum2(sv[q], cv[q], hi, lo);
+                put_pair(o, bf16, q, hi, lo);
+                if (K > 2) fin.see(hi);
+            };
+            auto pairs = [&](bool bf16) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float2 s = sv[q], c = cv[q];
-            if (want) {
-                if (A.out_bf16) {
-                    float2 hi, lo;
-                    two_sum2(s, c, hi, lo);
-                    put_pair(o, true, q, hi, lo);
-                    if (K > 2) fin.see(hi);
-                } else {
-                    const float2 hi = add2(s, c);
-                    put_pair(o, false, q, hi, hi);
-                    if (K > 2) fin.see(hi);
+                for (int q = 0; q < 4; ++q) pair(bf16, q);
+                put(u, bf16, o);
+            };
+            if constexpr (!GROUPED && K >= 5 && K != 7) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (A.out_bf16)
+                        pair(true, q);
+                    else
+                        pair(false, q);
                 }
+                put(u, A.out_bf16, o);
+            } else if (A.out_bf16) {
+                pairs(true);
+            } else {
+                pairs(false);
             }
-            if (accumulate) {
+        }
+        if (accumulate) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 s = sv[q], c = cv[q];
                 float2 x = make_float2(acc.x[u][2 * q], acc.x[u][2 * q + 1]);
                 float2 y = make_float2(acc.y[u][2 * q], acc.y[u][2 * q + 1]), e;
                 if constexpr (GATED) {
@@ -736,7 +761,6 @@ __device__ __forceinline__ void member_precise(const ExtrapArgs& A, bool want, c
                 acc.y[u][2 * q + 1] = y.y;
             }
         }
-        if (want) put(u, o);
     }
 }
 
@@ -751,26 +775,35 @@ __device__ __forceinline__ void resid_begin(Acc<UV>& acc, XLoad xload) {
     }
 }
 
-// Rounds the compensated hidden state to put(u, o), unless a result was not
+// Rounds the compensated hidden state to put(u, bf16, o), unless a result was not
 // finite (then nothing is stored and the caller recomputes the elements).
 template <int K, int UV, typename Put>
 __device__ __forceinline__ bool resid_precise(const ExtrapArgs& A, const Acc<UV>& acc, Finite& fin, Put put) {
-    uint32_t o[UV][8];
+    float2 hi[UV][4], lo[UV][4];
 #pragma unroll
     for (int u = 0; u < UV; ++u) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const float2 x = make_float2(acc.x[u][2 * q], acc.x[u][2 * q + 1]);
             const float2 y = make_float2(acc.y[u][2 * q], acc.y[u][2 * q + 1]);
-            float2 hi, lo;
-            two_sum2(x, y, hi, lo);
-            put_pair(o[u], A.resid_bf16, q, hi, lo);
-            if (K > 2) fin.see(hi);
+            two_sum2(x, y, hi[u][q], lo[u][q]);
+            if (K > 2) fin.see(hi[u][q]);
         }
     }
     if (K > 2 && !fin.all()) return false;
+    auto store = [&](bool bf16) {
 #pragma unroll
-    for (int u = 0; u < UV; ++u) put(u, o[u]);
+        for (int u = 0; u < UV; ++u) {
+            uint32_t o[8];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) put_pair(o, bf16, q, hi[u][q], lo[u][q]);
+            put(u, bf16, o);
+        }
+    };
+    if (A.resid_bf16)
+        store(true);
+    else
+        store(false);
     return true;
 }
 

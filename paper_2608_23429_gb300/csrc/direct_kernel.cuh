@@ -55,16 +55,16 @@ __device__ __forceinline__ void precise_vectors(const ExtrapArgs& A, int it, con
         void* out = member_out<K, CB16, UV>(A, first + m, ev, raw);
         float g[UV][8];
         if constexpr (GATED) load_gates<UV>(A, first + m, gi, g);
-        member_precise<K, CB16, UV, GATED>(
+        member_precise<K, CB16, UV, GATED, true>(
             A, out != nullptr, raw, resid != nullptr, acc, fin,
             [&](int u, float (&gv)[8]) {
 #pragma unroll
                 for (int e = 0; e < 8; ++e) gv[e] = g[u][e];
             },
-            [&](int u, const uint32_t (&o)[8]) { store_o8(out, A.out_bf16, ev[u], o); });
+            [&](int u, bool bf16, const uint32_t (&o)[8]) { store_o8(out, bf16, ev[u], o); });
     }
     if (resid ? !resid_precise<K, UV>(A, acc, fin,
-                                      [&](int u, const uint32_t (&o)[8]) { store_o8(resid, A.resid_bf16, ev[u], o); })
+                                      [&](int u, bool bf16, const uint32_t (&o)[8]) { store_o8(resid, bf16, ev[u], o); })
               : !fin.all())
         for (int u = 0; u < UV; ++u)
             for (int e = 0; e < kVecElems; ++e) scalar_element<CB16>(A, K, it, ev[u] + e);
