@@ -180,3 +180,35 @@ def test_steps_in_a_row_match_the_direct_kernel(cb, H, steps):
     for a, b in zip(got["auto"][0] + got["auto"][1], got["direct"][0] + got["direct"][1]):
         assert torch.equal(a.view(torch.int16), b.view(torch.int16))
     assert torch.equal(got["auto"][2], got["direct"][2])
+
+
+@pytest.mark.parametrize("gated", [False, True])
+@pytest.mark.parametrize("K,cache", [(6, "bf16"), (7, "bf16"), (6, "fp32")])
+def test_groups_too_large_to_hold(cb, H, K, cache, gated):
+    """Groups of four whose stages do not fit beside one another, whole tiles
+    and a ragged one: predictions and hidden states in bf16, on either side of
+    the rule that sends them to the compensated kernels."""
+    tensors = [workloads.TensorSpec(g, b, (2, 53, 136), g) for g in range(2) for b in range(4)]
+    w = workloads.Workload(name="deep", tensors=tensors, K=K, cache_dtype=cache, T=0, r=0, t_min=0.0, t_max=999.0,
+                           timesteps=[], degree=6, noise=0.1, seed=23)
+    nodes = [990.0 - 37.0 * k for k in range(K)]
+    walk = H.Walk(w, node_t=nodes)
+    cb.cb_plan_set_shapes(walk.plan, [s.shape for s in tensors])
+    for k, t in enumerate(nodes):
+        walk.push(t, k)
+    outs = [torch.empty(s.shape, dtype=torch.bfloat16, device="cuda") for s in tensors]
+    resid = [workloads.hidden_state(w, g, "cuda") for g in range(walk.n_groups)]
+    rh = [H.host(x) for x in resid]
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    gates = [torch.randn(s.shape[0], s.shape[2], generator=gen, device="cuda").bfloat16() for s in tensors]
+    target = nodes[-1] - 20.0
+    if gated:
+        cb.cb_extrapolate_gated(walk.plan, target, outs, cb.CB_BF16, resid, cb.CB_BF16, gates, cb.CB_BF16)
+    else:
+        cb.cb_extrapolate(walk.plan, target, outs, cb.CB_BF16, resid, cb.CB_BF16)
+    torch.cuda.synchronize()
+    assert cb.cb_plan_device_status(walk.plan) == 0
+    G = [H.expand_gate(g, s.shape) for g, s in zip(gates, tensors)] if gated else None
+    so, sr, _ = walk.expected_and_compare(target, outs, resid, rh, G=G)
+    assert so["bad"] == 0 and sr["bad"] == 0, (so, sr)
+    walk.close()
