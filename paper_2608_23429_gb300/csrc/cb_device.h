@@ -66,13 +66,13 @@ struct ExtrapArgs {
     long long slot_off[8];       // byte offset of history entry j (0 = oldest)
     float w_hi[8];               // fp32(w_j)
     float w_lo[8];               // fp32(w_j - w_hi[j])
-    float w_sum;                 // at least sum_j |w_hi[j]|
+    unsigned w_anchor[8];        // 2 |w_j|, rounded up: fp32, or bf16 twice for bf16 sources (see sum_vec)
     float w_guard[8];            // (K+2) u (1.01) 2^9 |w_hi[j]|: the fast path's scaled error bound
     int n_items;
     int tiles_total;
     int out_bf16;    // predictions are bf16 (else fp32)
     int resid_bf16;  // hidden states are bf16 (else fp32)
-    int precise;     // 1: compensated (Dot2) arithmetic for every element
+    int precise;     // 1: compensated arithmetic for every element
     int copy_out;    // full-step epilogue: outputs receive the (K = 1) sources converted, not a prediction
     int stages;                  // bulk variant: shared-memory pipeline depth
     unsigned stage_x_bytes;      // bulk variant: bytes of a tile's hidden state staged behind the K chunks (0: not staged)

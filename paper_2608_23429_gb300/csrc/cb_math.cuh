@@ -107,6 +107,12 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, pair_of(-1.0f), a); }  // a - b, rounded once
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// x y + z in bf16, both halves of a word
+__device__ __forceinline__ uint32_t fma_bf16x2(uint32_t x, uint32_t y, uint32_t z) {
+    uint32_t r;
+    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(y), "r"(z));
+    return r;
+}
 __device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
     s = add2(a, b);
     const float2 bb = sub2(s, a);
@@ -592,19 +598,29 @@ __device__ __forceinline__ void resid_fast(const ExtrapArgs& A, int it, const lo
 // 2q, 2q + 1 of one vector.
 //
 // K <= 2: Dot2 (its first TwoSum adds to zero and is left out). K >= 3: an
-// anchored sum. With M = 3 * 2^k, 2^k > W max_j |F_j| and W >= sum_j |w_hi[j]|,
-// every S_j = fl(w_hi[j] F_j + S_{j-1}), S_{-1} = M, stays in the binade of M,
-// so d_j = S_j - S_{j-1} is exact, and what the rounding left out,
-// w_hi[j] F_j - d_j (at most half a unit of M), is one FMA; c collects it with
-// the weight's low half. S_{K-1} - M is exact (the error-free extraction by a
-// large constant of Rump, Ogita & Oishi, "Accurate floating-point summation",
-// SIAM J. Sci. Comput. 31(1), 2008, with the product folded into the FMA).
-// Five operations per term against Dot2's eleven: with fp32 results the
-// kernels are bound by the FMA pipe. s + c is within 2^-40 sum_j |w_j F_j| of
-// the exact value (Dot2: 2^-45; 7e7 sums against quad precision, K = 3..8, bf16
-// and fp32 features), and the fp32 results' 2-norm error equals Dot2's to seven
-// digits.
-// Where M overflows (W max |F| >= 2^126) or a feature is not finite, s is not
+// anchored sum. With M >= 2 T, T = sum_j |w_hi[j] F_j|, every S_j =
+// fl(w_hi[j] F_j + S_{j-1}), S_{-1} = M, is at least T, so d_j = S_j - S_{j-1},
+// at most T, is exact, as is S_{K-1} - M; what the rounding left out, w_hi[j] F_j -
+// d_j, is one FMA, a second one adds the weight's low half to it, and c collects
+// the sum (the error-free extraction by a large constant of Rump, Ogita & Oishi,
+// "Accurate floating-point summation", SIAM J. Sci. Comput. 31(1), 2008, with the
+// product folded into the FMA).
+//
+// Error. With u = 2^-24, S_j <= (3 + small) T, so what is left out is at most
+// 3.3 u T each, and the roundings of its FMA, of the second one and of the K - 1
+// additions give |s + c - P| <= u^2 T (3.3 (K (K + 1) / 2 - 1) + 6.5 K): 2^-42 T
+// for K = 4, 2^-40.6 T for K = 8. Seen, over 2.9e7 sums against quad precision
+// (K = 3..8, bf16 and fp32 features, entries of one size and 2^30 apart, weights
+// of zero, cancelling terms): at most 2^-43.1 T, Dot2 2^-44.0 T; the fp32 results'
+// 2-norm error equals Dot2's to seven digits. An anchor from sum |w_j| times
+// max |F_j| is cheaper by an operation per term and no bound in T: a large
+// feature under a small weight takes the other terms' low bits (2^-22 T seen).
+//
+// Cost: seven operations per term of a pair (T is summed in bf16 for bf16 sources)
+// against Dot2's eleven: with fp32 results the kernels are bound by the FMA pipe
+// and the issue slots. The cheaper anchor measured DiT-XL/2 512^2, K = 8, fp32
+// predictions 734 us (737 us here) and K = 4 with gated fp32 hidden states 527 us (528).
+// Where M overflows (T >= 2^127) or a feature is not finite, s or c is not
 // finite: the callers then take scalar_element, which has no anchor.
 //
 // Two pairs advance together, term by term (four at once take registers from
@@ -637,29 +653,24 @@ __device__ __forceinline__ void sum_vec(const ExtrapArgs& A, const uint4 (&raw)[
         for (int q0 = 0; q0 < 4; q0 += 2) {
 #pragma unroll
             for (int q = q0; q < q0 + 2; ++q) {
-                float2 m;
-                if constexpr (CB16) {  // the signs of m are of no account: only its exponents are used
-                    uint32_t x = q == 0 ? raw[0][0].x : q == 1 ? raw[0][0].y : q == 2 ? raw[0][0].z : raw[0][0].w;
+                if constexpr (CB16) {
+                    uint32_t x = 0u;
 #pragma unroll
-                    for (int j = 1; j < K; ++j) {
+                    for (int j = 0; j < K; ++j) {
                         const uint4 v = raw[j][0];
-                        asm("max.xorsign.abs.bf16x2 %0, %0, %1;"
-                            : "+r"(x)
-                            : "r"(q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w));
+                        x = fma_bf16x2(A.w_anchor[j], (q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w) & 0x7FFF7FFFu, x);
                     }
-                    m = make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u));
+                    anchor[q] = make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u));
                 } else {
-                    m = vec_pair<CB16>(raw[0], q);
+                    float2 x = pair_of(0.0f);
 #pragma unroll
-                    for (int j = 1; j < K; ++j) {
+                    for (int j = 0; j < K; ++j) {
+                        const float w = __uint_as_float(A.w_anchor[j]);
                         const float2 f = vec_pair<CB16>(raw[j], q);
-                        m = make_float2(fmaxf(fabsf(m.x), fabsf(f.x)), fmaxf(fabsf(m.y), fabsf(f.y)));
+                        x = make_float2(fmaf(w, fabsf(f.x), x.x), fmaf(w, fabsf(f.y), x.y));
                     }
+                    anchor[q] = x;
                 }
-                const float2 v = mul2(pair_of(A.w_sum), m);
-                anchor[q] = mul2(make_float2(__uint_as_float(__float_as_uint(v.x) & 0x7F800000u),
-                                             __uint_as_float(__float_as_uint(v.y) & 0x7F800000u)),
-                                 pair_of(6.0f));
                 s[q] = anchor[q];
             }
 #pragma unroll
@@ -669,8 +680,8 @@ __device__ __forceinline__ void sum_vec(const ExtrapArgs& A, const uint4 (&raw)[
                 for (int q = q0; q < q0 + 2; ++q) {
                     const float2 f = vec_pair<CB16>(raw[j], q);
                     const float2 t = fma2(w, f, s[q]);
-                    const float2 r = fma2(w, f, sub2(s[q], t));
-                    c[q] = fma2(wl, f, j == 0 ? r : add2(c[q], r));
+                    const float2 r = fma2(wl, f, fma2(w, f, sub2(s[q], t)));
+                    c[q] = j == 0 ? r : add2(c[q], r);
                     s[q] = t;
                 }
             }

@@ -213,6 +213,18 @@ bool aligned(const void* ptr, size_t a) { return ((uintptr_t)ptr % a) == 0; }
 // Multiplier of the kernels' division by d < 2^32: ceil(2^64 / d), 0 for d <= 1.
 unsigned long long div_magic(unsigned d) { return d <= 1 ? 0ull : ~0ull / d + 1ull; }
 
+// 2 |w| as the compensated sums take it for their anchor (sum_vec): rounded up,
+// so far that K rounded additions cannot bring the sum below 2 sum_j |w_j F_j|.
+// fp32 for fp32 sources; for bf16 ones bf16, twice in one word.
+unsigned anchor_weight(double w, int K, bool src_bf16) {
+    const float x = (float)(2.0 * w * (1.0 + K * std::ldexp(1.0, src_bf16 ? -8 : -22)));
+    unsigned b;
+    std::memcpy(&b, &x, sizeof b);
+    if (!src_bf16) return b;
+    b = (b + 0xFFFFu) >> 16;  // up to the next bf16 (infinity past the largest)
+    return b << 16 | b;
+}
+
 // Logical history window: n entries, oldest first, with the slot of each.
 struct Window {
     int n;
@@ -598,18 +610,16 @@ int run_launch(cb_plan* p, const Window& win, const double* w, void* const* outs
     unsigned char* slot = p->cache + (size_t)p->next * p->slot_bytes;
     A.hist_base = feats ? 0ull : (unsigned long long)(uintptr_t)(ch ? ch->hist : p->cache);
     A.copy_out = feats ? 1 : 0;
-    double w_sum = 0.0;
     for (int j = 0; j < CB_MAX_K; ++j) {
         const bool on = j < K;
         A.slot_off[j] = on && !feats ? (long long)win.slot[j] * (long long)p->slot_bytes : 0;
         const float hi = on ? (float)w[j] : 0.0f;
         A.w_hi[j] = hi;
-        w_sum += std::fabs((double)hi);
         A.w_lo[j] = on ? (float)(w[j] - (double)hi) : 0.0f;
         // the fast path's bound, scaled: (K+2) u (1.01) 2^9 |w_hi[j]|, u = 2^-24
         A.w_guard[j] = (float)(std::fabs((double)hi) * (K + 2) * 1.01 * std::ldexp(1.0, -15));
+        A.w_anchor[j] = anchor_weight(std::fabs((double)hi), K, cb16);
     }
-    A.w_sum = std::nextafterf((float)w_sum, INFINITY);
     A.out_bf16 = out_dtype == CB_BF16;
     A.resid_bf16 = resid_dtype == CB_BF16;
 

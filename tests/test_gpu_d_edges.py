@@ -212,3 +212,53 @@ def test_groups_too_large_to_hold(cb, H, K, cache, gated):
     so, sr, _ = walk.expected_and_compare(target, outs, resid, rh, G=G)
     assert so["bad"] == 0 and sr["bad"] == 0, (so, sr)
     walk.close()
+
+
+@pytest.mark.parametrize("kernel", ["bulk", "direct"])
+@pytest.mark.parametrize("K,cache,io", [(3, "bf16", "fp32"), (4, "bf16", "bf16"), (8, "bf16", "fp32"), (3, "fp32", "bf16"),
+                                        (5, "fp32", "fp32"), (8, "fp32", "fp32")])
+@pytest.mark.parametrize("weight", [0.0, 2.0 ** -24])
+def test_a_large_feature_under_a_small_weight(cb, H, K, cache, io, kernel, weight):
+    """One history entry 2^20 to 2^30 times the size of the others, with a weight
+    of (nearly) nothing, and the others' terms cancelling to any depth: whole
+    tiles, a ragged one, and buffers off the 16-byte grid. The error bound of the
+    compensated sums is u |P| + 2^-40 sum_j |w_j F_j| for fp32 results (u = 2^-24,
+    one rounding) and the bf16 gate's otherwise."""
+    sizes = [9728, 6099, 4865]
+    tensors = [workloads.TensorSpec(i, 0, (1, 1, n), i) for i, n in enumerate(sizes)]
+    w = workloads.Workload(name="spread", tensors=tensors, K=K, cache_dtype=cache, T=0, r=0, t_min=0.0, t_max=999.0,
+                           timesteps=[], degree=1, noise=0.0, seed=1)
+    nodes = [900.0 - 50.0 * k for k in range(K)]
+    walk = H.Walk(w, node_t=nodes, kernel=kernel)
+    rng = np.random.default_rng(12 + K)
+    wts = rng.standard_normal(K)
+    wts[K // 2] = weight
+    feats = [[None] * len(sizes) for _ in range(K)]
+    for i, n in enumerate(sizes):
+        f = rng.standard_normal((K, n))
+        f[K // 2] *= 2.0 ** rng.uniform(20, 30, n)
+        rest = sum(wts[j] * f[j] for j in range(1, K) if j != K // 2)
+        f[0] = -rest / wts[0] * (1 + rng.standard_normal(n) * 2.0 ** -rng.uniform(0, 20, n))
+        for j in range(K):
+            feats[j][i] = torch.tensor(f[j], device="cuda").to(H.TORCH[cache])
+    for j in range(K):
+        cb.cb_cache_push(walk.plan, feats[j], H.CB[cache], nodes[j])
+    dt = H.TORCH[io]
+    outs, resid = [[_shifted((1, 1, n), dt, int(i == 2))[0] for i, n in enumerate(sizes)] for _ in range(2)]
+    for x in resid:
+        x.copy_(torch.tensor(rng.standard_normal(x.shape) * 2.0 ** -8))
+    x64 = [x.double().cpu().numpy().reshape(-1) for x in resid]
+    cb.cb_extrapolate_weights(walk.plan, wts, outs, H.CB[io], resid, H.CB[io])
+    torch.cuda.synchronize()
+    assert cb.cb_plan_device_status(walk.plan) == 0
+    for i in range(len(sizes)):
+        f64 = np.array([feats[j][i].double().cpu().numpy() for j in range(K)])
+        p, bound = wts @ f64, np.abs(wts) @ np.abs(f64)
+        for got, want, b in [(outs[i], p, bound), (resid[i], p + x64[i], bound + np.abs(x64[i]))]:
+            if io == "bf16":
+                st = H.compare_bf16(H.host(got), orc.convert(want, orc.FP64, orc.BF16), want, b)
+                assert st["bad"] == 0, (i, st)
+            else:
+                err = np.abs(H.host(got).astype(np.float64) - want)
+                assert np.all(err <= 2.0 ** -24 * np.abs(want) + H.FLOOR * b), (i, float((err / b).max()))
+    walk.close()
