@@ -35,7 +35,9 @@ cudaError_t launch_overlapped(void (*kernel)(Args), int grid, int threads, size_
     c.attrs = &at;
     c.numAttrs = 1;
     void* args[] = {const_cast<void*>(static_cast<const void*>(&a))};
-    return cudaLaunchKernelExC(&c, reinterpret_cast<const void*>(kernel), args);
+    const cudaError_t e = cudaLaunchKernelExC(&c, reinterpret_cast<const void*>(kernel), args);
+    if (e != cudaSuccess) (void)cudaGetLastError();  // returned here, so not left for a check of the caller's own launches
+    return e;
 }
 
 #ifdef __CUDACC__

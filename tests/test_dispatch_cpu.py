@@ -1,0 +1,70 @@
+"""Which kernel a call runs, with what, and what stays behind when a launch fails:
+the library's host side over stand-ins for the CUDA runtime and the launchers
+(host_stub.cpp), on the CPU."""
+import ctypes
+import importlib.util
+import os
+import re
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+NODES = [900.0 - 50.0 * k for k in range(8)]
+
+
+@pytest.fixture(scope="module")
+def cb(tmp_path_factory):
+    """The binding over the stub, with `stub` for the stub's own functions."""
+    from paper_2608_23429_gb300 import build
+    build.build()
+    so = str(tmp_path_factory.mktemp("stub") / "libstub.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")
+    subprocess.run([shutil.which("g++"), "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", f"-I{cuda}", "-o", so,
+                    os.path.join(ROOT, "tests", "host_stub.cpp"), os.path.join(build.CSRC, "plan.cpp")], check=True)
+    spec = importlib.util.spec_from_file_location("chebboost_on_stub", os.path.join(build.HERE, "chebboost.py"))
+    mod = importlib.util.module_from_spec(spec)
+    cdll, ctypes.CDLL = ctypes.CDLL, lambda path, *a: cdll(so)
+    try:
+        spec.loader.exec_module(mod)
+    finally:
+        ctypes.CDLL = cdll
+    mod.stub = cdll(so)
+    mod.stub.stub_log.restype = ctypes.c_char_p
+    return mod
+
+
+def _log(cb):
+    """(name, {field: value}) of every call noted since the last reset."""
+    return [(line.split()[0], {k: int(v) for k, v in re.findall(r"(\w+)=(\d+)", line)})
+            for line in cb.stub.stub_log().decode().splitlines()]
+
+
+def _plan(cb, K, shapes, groups, cache, steps=None):
+    plan = cb.cb_plan_create(NODES[:max(K, 1)], K, [(i, 0, b * t * h, g) for i, ((b, t, h), g) in enumerate(zip(shapes, groups))],
+                             cache, 0.0, 999.0)
+    cb.cb_plan_set_shapes(plan, shapes)
+    cb.cb_plan_bind_cache(plan, 1 << 40, cb.cb_plan_cache_bytes(plan))
+    cb.stub.stub_reset()
+    for k in range(K if steps is None else steps):
+        cb.cb_cache_push(plan, [(1 << 41) + (i << 32) for i in range(len(shapes))], cache, NODES[k])
+    cb.stub.stub_reset()
+    return plan
+
+
+def _addresses(n, base, off=0):
+    return [base + (i << 32) + off for i in range(n)]
+
+
+def test_failed_launch_leaves_no_error_behind(cb):
+    """A launch that fails reports CB_ERR_CUDA once: the runtime's last error is
+    taken with it, so that the caller's next check finds none."""
+    plan = _plan(cb, 3, [(1, 16, 64)], [-1], cb.CB_BF16, steps=1)
+    cb.stub.stub_fail(b"launch")
+    with pytest.raises(cb.CbError) as e:
+        cb.cb_cache_push(plan, [1 << 41], cb.CB_BF16, NODES[1])
+    assert e.value.status == cb.CB_ERR_CUDA
+    assert cb.stub.stub_last_error() == 0
+    cb.cb_cache_push(plan, [1 << 41], cb.CB_BF16, NODES[1])  # the failed step left the history as it was
+    cb.cb_plan_destroy(plan)
