@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -312,13 +313,18 @@ int clear_status_once(cb_plan* p, void* stream) {
 }
 
 // A history buffer given with the call instead of the bound arena, and the
-// status word its launches record into (cb_extrapolate_noalloc; null: none).
-// `launched` is set once a launch is under way.
+// status word of device `device` its launches record into (cb_extrapolate_noalloc;
+// null: none). `launched` is set once a launch is under way.
 struct CallerHistory {
     const unsigned char* hist;
     int* status;
+    int device;
     bool launched;
 };
+
+// Devices whose no-alloc status word may hold a code that nobody was told: a
+// call failed between its launch and the handover that clears the word.
+std::atomic<bool> g_unclaimed[cbk::kMaxStatusDevices];
 
 // What the launches of one call share.
 struct Launch {
@@ -333,8 +339,19 @@ struct Launch {
 };
 
 int clear_status(Launch& L) {
-    if (!L.ch) return clear_status_once(L.p, L.stream);
-    L.ch->launched = true;  // that word is zero (static_status.cu)
+    CallerHistory* ch = L.ch;
+    if (!ch) return clear_status_once(L.p, L.stream);
+    // Its word is zero, but for what a failed call left there. A clearing that is
+    // captured runs later: the word stays unclaimed until one has been enqueued.
+    if (ch->status && !ch->launched && g_unclaimed[ch->device]) {
+        const cudaStream_t s = (cudaStream_t)L.stream;
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(s, &capture);
+        if (e == cudaSuccess) e = cudaMemsetAsync(ch->status, 0, sizeof(int), s);
+        if (e != cudaSuccess) return cuda_fail(e, "status word");
+        if (capture == cudaStreamCaptureStatusNone) g_unclaimed[ch->device] = false;
+    }
+    ch->launched = true;
     return CB_OK;
 }
 
@@ -921,9 +938,11 @@ int cb_extrapolate_noalloc(cb_plan* p, const void* hist, size_t hist_bytes, cons
     e = cbk::noalloc_status_word(dev, &word);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress");
     // Only launches whose status is asked for record into the word, and handing
-    // it over clears it, so that it needs no clearing before a launch.
-    CallerHistory ch{static_cast<const unsigned char*>(hist), status ? word : nullptr, false};
+    // it over clears it, so that it needs no clearing before a launch (unless a
+    // call failed in between: clear_status).
+    CallerHistory ch{static_cast<const unsigned char*>(hist), status ? word : nullptr, dev, false};
     rc = run_launch(p, win, w, outs, out_dtype, resid, resid_dtype, stream, nullptr, CB_BF16, nullptr, CB_BF16, &ch);
+    if (rc != CB_OK && status && ch.launched) g_unclaimed[dev] = true;
     if (rc != CB_OK || !status) return rc;
     if (!ch.launched) {  // nothing was requested, so nothing ran
         *status = 0;
@@ -939,7 +958,10 @@ int cb_extrapolate_noalloc(cb_plan* p, const void* hist, size_t hist_bytes, cons
         e = cudaMemcpyAsync(status, word, sizeof(int), cudaMemcpyDeviceToHost, (cudaStream_t)stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(word, 0, sizeof(int), (cudaStream_t)stream);
     }
-    if (e != cudaSuccess) return cuda_fail(e, "status read-back");
+    if (e != cudaSuccess) {
+        g_unclaimed[dev] = true;
+        return cuda_fail(e, "status read-back");
+    }
     return CB_OK;
 }
 

@@ -68,3 +68,41 @@ def test_failed_launch_leaves_no_error_behind(cb):
     assert cb.stub.stub_last_error() == 0
     cb.cb_cache_push(plan, [1 << 41], cb.CB_BF16, NODES[1])  # the failed step left the history as it was
     cb.cb_plan_destroy(plan)
+
+
+def _noalloc(cb, plan, outs, status):
+    n = cb.cb_plan_cache_bytes(plan) - cb.CB_STATUS_BYTES
+    cb.cb_extrapolate_noalloc(plan, 1 << 42, n, NODES[:3], 0, 780.0, outs, cb.CB_BF16, status=status)
+
+
+@pytest.mark.parametrize("fails", ["bulk", "bulk_strided", "take_status", "memcpy", "memset"])
+def test_status_that_nobody_was_told_is_cleared(cb, fails):
+    """A call that fails between its launch and the handover of the status word
+    leaves that word to be cleared by the next call that asks, once, before its
+    launch; a captured clearing runs later and does not count."""
+    plan = _plan(cb, 3, [(1, 64, 64)] * 2, [-1, -1], cb.CB_BF16)
+    outs = [(1 << 43) + 16, (1 << 44) + 2]  # an aligned one and one off the grid: two launches
+    word = ctypes.c_int(-1)
+    pinned = fails not in ("memcpy", "memset")
+    cb.stub.stub_host_memory(pinned)
+    cb.stub.stub_fail(fails.encode())
+    with pytest.raises(cb.CbError):
+        _noalloc(cb, plan, outs, ctypes.addressof(word))
+
+    def calls(status):
+        cb.stub.stub_reset()
+        cb.stub.stub_host_memory(1)
+        return_to = ctypes.addressof(word) if status else None
+        _noalloc(cb, plan, outs, return_to)
+        return [c[0] for c in _log(cb)]
+
+    launches = ["bulk_strided", "bulk"]
+    assert calls(False) == launches  # asks nothing, records nothing
+    cb.stub.stub_reset()
+    cb.stub.stub_host_memory(1)
+    cb.stub.stub_capturing(1)
+    _noalloc(cb, plan, outs, ctypes.addressof(word))
+    assert [c[0] for c in _log(cb)] == ["memset"] + launches + ["take_status"]
+    assert calls(True) == ["memset"] + launches + ["take_status"]
+    assert calls(True) == launches + ["take_status"]
+    cb.cb_plan_destroy(plan)
