@@ -951,7 +951,7 @@ int cb_extrapolate_noalloc(cb_plan* p, const void* hist, size_t hist_bytes, cons
     cudaPointerAttributes at{};
     const bool pinned = cudaPointerGetAttributes(&at, status) == cudaSuccess && at.type == cudaMemoryTypeHost &&
                         at.devicePointer != nullptr;
-    if (pinned) {
+    if (pinned && aligned(at.devicePointer, sizeof(int))) {  // a kernel's store wants the alignment, a copy does not
         e = cbk::take_status(word, static_cast<int*>(at.devicePointer), (cudaStream_t)stream);
     } else {
         (void)cudaGetLastError();  // a pointer the runtime does not know is ordinary memory

@@ -106,3 +106,15 @@ def test_status_that_nobody_was_told_is_cleared(cb, fails):
     assert calls(True) == ["memset"] + launches + ["take_status"]
     assert calls(True) == launches + ["take_status"]
     cb.cb_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2])
+def test_status_off_the_word_grid_is_copied(cb, offset):
+    """The device writes a pinned status itself only where an int may lie; any
+    other address is copied to, as ordinary memory is."""
+    plan = _plan(cb, 3, [(1, 64, 64)], [-1], cb.CB_BF16)
+    buf = (ctypes.c_int * 2)()
+    cb.stub.stub_host_memory(1)
+    _noalloc(cb, plan, [1 << 43], ctypes.addressof(buf) + offset)
+    assert [c[0] for c in _log(cb)] == ["bulk"] + (["take_status"] if offset == 0 else ["memcpy", "memset"])
+    cb.cb_plan_destroy(plan)
