@@ -188,7 +188,8 @@ __device__ __forceinline__ void produce(const ExtrapArgs& A, uint32_t full0, uin
 }
 
 // Elements i, i + 1 of a ragged tile (n elements, of which the first `staged`
-// lie in the chunk at p) as words of a vector; zero past the end.
+// lie in the chunk at p) as words of a vector. A tensor of odd length ends inside
+// a pair: its second half is then whatever the slot's padding holds (no_padding).
 // TAIL: some elements may not be staged (a full step's new features).
 template <bool CB16, bool TAIL>
 __device__ __forceinline__ uint2 ragged_pair(const unsigned char* p, int i, int n, int staged,
@@ -208,6 +209,27 @@ __device__ __forceinline__ uint2 ragged_pair(const unsigned char* p, int i, int 
         w = make_uint2(q[0], i + 1 < n ? q[1] : 0u);
     }
     return w;
+}
+
+// Clears the second half of the pair that ends a tensor of odd length n, in the
+// history values of the vector whose pair q begins at at(q): the padding is
+// nobody's value, and a NaN there would decide how the thread's other elements
+// are summed. Once per vector, behind a branch that tiles of even length skip:
+// tested with each pair's load it cost the fp32 kernels 14 to 40 registers.
+template <int K, bool CB16, typename At>
+__device__ __forceinline__ void no_padding(uint4 (&raw)[K][CB16 ? 1 : 2], int n, At at) {
+    if ((n & 1) == 0) return;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (at(q) + 1 != n) continue;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            if constexpr (CB16)
+                (q == 0 ? raw[j][0].x : q == 1 ? raw[j][0].y : q == 2 ? raw[j][0].z : raw[j][0].w) &= 0xFFFFu;
+            else
+                ((q & 1) ? raw[j][q >> 1].w : raw[j][q >> 1].y) = 0u;
+        }
+    }
 }
 
 // Four pairs of elements p[at(q, 0)], p[at(q, 1)]; 0 where in(q, e) is false.
@@ -362,6 +384,9 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
                     }
                 }
             }
+        if constexpr (RAGGED && !FULL)
+#pragma unroll
+            for (int v = 0; v < U; ++v) no_padding<K, CB16>(raw[v], n, [&](int q) { return pair_at(v, q); });
         if constexpr (STAGED_GATES) {  // rows that came with the stage, or from global memory
             const void* gp = gated ? A.m_gate[first + m] : nullptr;
             if (gp != nullptr && A.stage_gate_bytes) gp = base + K * Sh::chunk + A.stage_x_bytes;

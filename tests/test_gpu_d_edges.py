@@ -262,3 +262,36 @@ def test_a_large_feature_under_a_small_weight(cb, H, K, cache, io, kernel, weigh
                 err = np.abs(H.host(got).astype(np.float64) - want)
                 assert np.all(err <= 2.0 ** -24 * np.abs(want) + H.FLOOR * b), (i, float((err / b).max()))
     walk.close()
+
+
+@pytest.mark.parametrize("cache", ["bf16", "fp32"])
+def test_slot_padding_does_not_matter(cb, H, cache):
+    """Tensors of odd length, whose last pair ends in the slot's padding: the
+    same bits whether that holds zeros or NaN, with terms that cancel so far that
+    another way of summing would show."""
+    K, sizes = 8, [2501 + 2 * i for i in range(40)]
+    tensors = [workloads.TensorSpec(i, 0, (1, 1, n), -1) for i, n in enumerate(sizes)]
+    w = workloads.Workload(name="padding", tensors=tensors, K=K, cache_dtype=cache, T=0, r=0, t_min=0.0, t_max=999.0,
+                           timesteps=[], degree=1, noise=0.0, seed=1)
+    nodes = [900.0 - 50.0 * k for k in range(K)]
+    rng = np.random.default_rng(4)
+    wts = rng.standard_normal(K)
+    feats = [[None] * len(sizes) for _ in range(K)]
+    for i, n in enumerate(sizes):
+        f = rng.standard_normal((K, n))
+        f[0] = -(wts[1:] @ f[1:]) / wts[0] * (1 + rng.standard_normal(n) * 2.0 ** -26)
+        for j in range(K):
+            feats[j][i] = torch.tensor(f[j], device="cuda").to(H.TORCH[cache])
+    got = []
+    for fill in (0x00, 0xFF):
+        walk = H.Walk(w, node_t=nodes, kernel="bulk")
+        walk.cache.fill_(fill)
+        for j in range(K):
+            cb.cb_cache_push(walk.plan, feats[j], H.CB[cache], nodes[j])
+        outs = [torch.empty(n, dtype=torch.float32, device="cuda") for n in sizes]
+        cb.cb_extrapolate_weights(walk.plan, wts, outs, cb.CB_FP32)
+        torch.cuda.synchronize()
+        assert cb.cb_plan_device_status(walk.plan) == 0
+        got.append(outs)
+        walk.close()
+    assert all(torch.equal(a, b) for a, b in zip(*got))
