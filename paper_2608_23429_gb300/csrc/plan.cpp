@@ -479,12 +479,22 @@ int launch_bulk(Launch& L, cbk::ExtrapArgs& A, bool strided) {
         }
         if (fits && need <= kMaxStagedGateBytes) A.stage_gate_bytes = (unsigned)((need + 127) / 128 * 128);
     }
-    size_t smem = 0;
+    size_t smem = 0, stage_bytes = 0;
     int per_sm = 1;
-    const size_t stage_bytes =
-        (size_t)K * shape.tile * esize(cb16 ? CB_BF16 : CB_FP32) + A.stage_x_bytes + A.stage_gate_bytes;
-    rc = bulk_config(p, K, cb16, gated, precise, strided, shape.ctas_per_sm, stage_bytes, min_stages, &A.stages, &smem,
-                     &per_sm);
+    auto fit = [&] {
+        stage_bytes = (size_t)K * shape.tile * esize(cb16 ? CB_BF16 : CB_FP32) + A.stage_x_bytes + A.stage_gate_bytes;
+        return bulk_config(p, K, cb16, gated, precise, strided, shape.ctas_per_sm, stage_bytes, min_stages, &A.stages,
+                           &smem, &per_sm);
+    };
+    rc = fit();
+    // Gate rows too wide to lie beside the stages stay in global memory, rather than
+    // that another kernel runs (GB300, [1, 4096, 3072], fp32 gates, direct kernel ->
+    // here: fp32 sources, K = 8, groups of one 418 -> 288 us, of two 691 -> 512 us;
+    // bf16 groups of two, K = 6 573 -> 520 us).
+    if (rc == CB_OK && A.stages < min_stages && A.stage_gate_bytes) {
+        A.stage_gate_bytes = 0;
+        rc = fit();
+    }
     if (rc != CB_OK) return rc;
     if (A.stages < min_stages) {  // too deep for shared memory
         // A group too large to hold: the compensated kernels hold none (GB300,

@@ -118,3 +118,18 @@ def test_status_off_the_word_grid_is_copied(cb, offset):
     _noalloc(cb, plan, [1 << 43], ctypes.addressof(buf) + offset)
     assert [c[0] for c in _log(cb)] == ["bulk"] + (["take_status"] if offset == 0 else ["memcpy", "memset"])
     cb.cb_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("K,cache,io,gate,members,hidden,name,staged",
+                         [(8, 1, 1, 1, 1, 1024, "bulk_precise", True), (8, 1, 1, 1, 1, 2048, "bulk_precise", False),
+                          (8, 1, 1, 0, 2, 4096, "bulk_precise", False), (5, 0, 0, 1, 2, 3072, "bulk_gated", True),
+                          (6, 0, 0, 1, 2, 3072, "bulk_gated", False), (2, 0, 1, 1, 2, 4096, "bulk_precise", True)])
+def test_wide_gate_rows_stay_on_the_pipeline(cb, K, cache, io, gate, members, hidden, name, staged):
+    """Gate rows that leave no room for the pipeline's stages are left in global
+    memory; the launch keeps its kernel."""
+    plan = _plan(cb, K, [(1, 64, hidden)] * members, [0] * members, cache)
+    cb.cb_extrapolate_gated(plan, 100.0, None, io, [1 << 45], io, _addresses(members, 1 << 43), gate)
+    (got, a), = _log(cb)
+    assert got == name and (a["gates"] > 0) == staged and a["stages"] >= (2 if name == "bulk_precise" else members + 1), a
+    assert a["smem"] <= 232448
+    cb.cb_plan_destroy(plan)

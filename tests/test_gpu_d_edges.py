@@ -295,3 +295,30 @@ def test_slot_padding_does_not_matter(cb, H, cache):
         got.append(outs)
         walk.close()
     assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+@pytest.mark.parametrize("K,cache,io,members,hidden", [(8, "fp32", "fp32", 1, 2048), (6, "bf16", "bf16", 2, 3072)])
+def test_wide_gate_rows(cb, H, K, cache, io, members, hidden):
+    """fp32 gate rows too wide to be staged beside the pipeline's stages, read from
+    global memory by the same kernels: two batches, whole tiles and a ragged one."""
+    tensors = [workloads.TensorSpec(g, b, (2, 13, hidden), g) for g in range(2) for b in range(members)]
+    w = workloads.Workload(name="wide", tensors=tensors, K=K, cache_dtype=cache, T=0, r=0, t_min=0.0, t_max=999.0,
+                           timesteps=[], degree=6, noise=0.1, seed=29)
+    nodes = [990.0 - 37.0 * k for k in range(K)]
+    walk = H.Walk(w, node_t=nodes)
+    cb.cb_plan_set_shapes(walk.plan, [s.shape for s in tensors])
+    for k, t in enumerate(nodes):
+        walk.push(t, k)
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    gates = [torch.randn(s.shape[0], s.shape[2], generator=gen, device="cuda") for s in tensors]
+    resid = [workloads.hidden_state(w, g, "cuda", H.TORCH[io]) for g in range(walk.n_groups)]
+    rh = [H.host(x) for x in resid]
+    outs = [torch.empty(s.shape, dtype=H.TORCH[io], device="cuda") for s in tensors]
+    target = nodes[-1] - 20.0
+    cb.cb_extrapolate_gated(walk.plan, target, outs, H.CB[io], resid, H.CB[io], gates, cb.CB_FP32)
+    torch.cuda.synchronize()
+    assert cb.cb_plan_device_status(walk.plan) == 0
+    G = [H.expand_gate(g, s.shape) for g, s in zip(gates, tensors)]
+    so, sr, _ = walk.expected_and_compare(target, outs, resid, rh, out_dtype=io, resid_dtype=io, G=G)
+    assert so["bad"] == 0 and sr["bad"] == 0, (so, sr)
+    walk.close()
