@@ -570,12 +570,16 @@ int launch_bulk(Launch& L, cbk::ExtrapArgs& A, bool strided) {
         const double l2 = p->dev.l2_bytes, room = 0.4 * l2;
         if (rd + wr > room && wr <= 0.55 * l2) A.keep_tiles = (int)(std::max(0.0, room - wr) / rd * A.tiles_total);
     }
-    // The gated one-entry epilogue cannot hold two groups of two and keep to its
-    // bytes in flight: a twentieth of the SMs less does it (GB300, groups of
-    // two, [8, 256, 1152], [4, 1024, 1152], [2, 4096, 1152] and [1, 4096, 3072]:
-    // 128.5 -> 125.2, 250 -> 246, 493 -> 486, 658 -> 651 us; groups of one and
-    // three and fp32 gates lose 1 to 4 % by it).
-    if (L.full_step && cb16 && gated && hold && max_nb == 2 && L.gate_dtype == CB_BF16) frac = 0.95;
+    // The gated one-entry epilogue of bf16 groups of two holds more in flight than
+    // the mix wants: a twentieth of the SMs less pays where a launch is long and its
+    // gate rows narrow (GB300, tiles per SM 53, 71, 106, 189, 212: 66.1 -> 65.8, 85.9 ->
+    // 84.4, 126.0 -> 124.9, 218.6 -> 215.6, 246 -> 243 us). Short launches lose their
+    // overlap by it (0.5, 4, 8, 40 tiles per SM 4.8 -> 6.2, 7.2 -> 8.2, 13.2 -> 14.4, 51.1
+    // -> 51.3 us), rows of 3072 channels 0.5 to 3 % (146 -> 150, 641 -> 646 us), groups of
+    // one and three and fp32 gates 1 to 4 %.
+    if (L.full_step && cb16 && gated && hold && max_nb == 2 && L.gate_dtype == CB_BF16 &&
+        A.stage_gate_bytes <= 8192 && A.tiles_total >= 48LL * p->dev.sms)
+        frac = 0.95;
     const long long ctas = std::max(1LL, (long long)((double)p->dev.sms * per_sm * frac));
     // An overlapping launch's blocks go wherever they fit: ask for so much shared
     // memory that no SM takes more than its share of them.

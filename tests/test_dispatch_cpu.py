@@ -133,3 +133,19 @@ def test_wide_gate_rows_stay_on_the_pipeline(cb, K, cache, io, gate, members, hi
     assert got == name and (a["gates"] > 0) == staged and a["stages"] >= (2 if name == "bulk_precise" else members + 1), a
     assert a["smem"] <= 232448
     cb.cb_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("groups,batch,tokens,hidden,fewer", [(1, 1, 256, 1152, False), (28, 1, 256, 1152, False),
+                                                              (4, 4, 1024, 1152, False), (28, 8, 256, 1152, True),
+                                                              (28, 4, 1024, 2048, True), (19, 1, 4096, 3072, False)])
+def test_gated_full_steps_take_every_processor_unless_large(cb, groups, batch, tokens, hidden, fewer):
+    """Gated full steps of groups of two: a launch that leaves processors free
+    cannot overlap the one before, which small steps live by."""
+    plan = _plan(cb, 3, [(batch, tokens, hidden)] * (2 * groups), [i // 2 for i in range(2 * groups)], cb.CB_BF16, steps=0)
+    cb.cb_cache_push_residual(plan, _addresses(2 * groups, 1 << 41), cb.CB_BF16, NODES[0], _addresses(groups, 1 << 42),
+                              cb.CB_BF16, _addresses(2 * groups, 1 << 43), cb.CB_BF16)
+    (name, a), = [c for c in _log(cb) if c[0] != "memset"]
+    tiles = groups * batch * tokens * hidden // 4096
+    assert name == "bulk_gated" and a["overlap"] == int(not fewer)
+    assert a["grid"] == (288 if fewer else min(304, tiles))
+    cb.cb_plan_destroy(plan)
