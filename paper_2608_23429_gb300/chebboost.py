@@ -107,7 +107,7 @@ def ptr_array(xs):
     try:
         addrs = [x.data_ptr() for x in xs]
     except AttributeError:  # addresses or None among them
-        addrs = [_addr(x) or 0 for x in xs]
+        addrs = [(_addr(x) or 0) & 0xFFFFFFFFFFFFFFFF for x in xs]  # as ctypes takes them, signed ones too
     return (ctypes.c_void_p * len(xs)).from_buffer(array("Q", addrs))
 
 

@@ -337,3 +337,19 @@ def test_short_weight_vector_is_rejected_not_overread(cb):
     assert buf.size == cb.CB_MAX_K and buf[0] == 0.5 and np.isnan(buf[1:]).all()
     cb.cb_plan_destroy(p)
     assert cb._dims(p) is None
+
+
+@pytest.mark.parametrize("xs", [[], [None, 0x1000], [-4096, 1 << 63, None], [np.zeros(1), 0x20, None]])
+def test_pointer_arrays_hold_the_addresses_ctypes_would(cb, xs):
+    """Addresses as integers of either sign, buffers, None, and none at all."""
+    class Buffer:
+        def __init__(self, x):
+            self.x = x
+
+        def data_ptr(self):
+            return self.x.ctypes.data
+
+    xs = [Buffer(x) if isinstance(x, np.ndarray) else x for x in xs]
+    want = (ctypes.c_void_p * len(xs))(*[x.data_ptr() if isinstance(x, Buffer) else x for x in xs])
+    got = cb.ptr_array(xs)
+    assert type(got) is type(want) and list(got) == list(want)
