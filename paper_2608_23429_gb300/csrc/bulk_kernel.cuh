@@ -400,12 +400,7 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
             }
         }
         if (GROUPED && !RAGGED && m == 0 && resid != nullptr)
-            resid_begin<U>(acc, [&](int v, float (&x)[8]) {
-                if (A.stage_x_bytes)
-                    load_x8(base + K * Sh::chunk, A.resid_bf16, at(v), x);
-                else
-                    load_x8(resid, A.resid_bf16, e0 + at(v), x);
-            });
+            resid_begin<U>(acc, [&](int v, float (&x)[8]) { load_x8(base + K * Sh::chunk, A.resid_bf16, at(v), x); });
         release_stage(empty0 + 8u * stage, lane);
         void* out = A.m_out[first + m];
         bool want = out != nullptr;

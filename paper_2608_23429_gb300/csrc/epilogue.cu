@@ -33,50 +33,32 @@ static_assert(epilogue_tile_elems == (long long)kThreads * kVecElems, "one vecto
 
 // One 8-element vector (element ev[0]) of item `it` through every member and
 // the hidden state.
-template <bool CB16, bool GATED>
 __device__ __forceinline__ void epilogue_vector(const ExtrapArgs& A, int it, const long long (&ev)[1]) {
     const int nb = A.nb[it];
     const int first = A.first[it];
     void* resid = A.resid[it];
     // loads first: every member's features and the bf16 hidden state
-    RawVecs<1, CB16, 1> raw[kEpilogueMaxMembers];
+    RawVecs<1, true, 1> raw[kEpilogueMaxMembers];
 #pragma unroll
     for (int m = 0; m < kEpilogueMaxMembers; ++m)
-        if (m < nb) load_member<1, CB16, 1>(A, A.m_off[first + m], ev, raw[m]);
+        if (m < nb) load_member<1, true, 1>(A, A.m_off[first + m], ev, raw[m]);
     uint4 xr = make_uint4(0u, 0u, 0u, 0u);
     if (resid) xr = ld_v4(reinterpret_cast<const unsigned char*>(resid) + ev[0] * 2);
-    unsigned gi[1] = {0u};
-    if constexpr (GATED) {  // items without shapes carry no gate
-        if (resid && A.i_hidden[it] != 0) gate_offsets<1>(A, it, ev[0], ev, gi);
-    }
     Acc<1> acc;
     acc.zero();
 #pragma unroll
     for (int m = 0; m < kEpilogueMaxMembers; ++m) {
         if (m >= nb) break;
-        member_out<1, CB16, 1>(A, first + m, ev, raw[m]);  // the slot write
-        if (!resid) continue;
-        const void* gp = GATED ? A.m_gate[first + m] : nullptr;
-        auto gate = [&](int, float (&gv)[8]) {
-            if (gp)
-                load_x8(gp, A.gate_bf16, (long long)gi[0], gv);
-            else
-#pragma unroll
-                for (int e = 0; e < 8; ++e) gv[e] = 1.0f;
-        };
-        if constexpr (CB16)  // bf16 features: exact, no weighted sum
-            member_one<1, CB16, 1, GATED>(raw[m], acc, gate);
-        else
-            member_fast<1, CB16, 1, false, GATED>(A, A.m_off[first + m], nullptr, ev, raw[m], true, acc, gate);
+        member_out<1, true, 1>(A, first + m, ev, raw[m]);  // the slot write
+        if (resid) member_one<1, true, 1>(raw[m], acc);    // bf16 features: exact, no weighted sum
     }
     if (!resid) return;
     resid_fast<1, 1>(
         A, it, ev, acc, resid, [&](int, float (&x)[8]) { unpack_bf16x8(xr, x); },
-        [&](int, int e, float xe, float& hi, float& lo) { exact_resid<CB16>(A, 1, it, ev[0] + e, xe, hi, lo); },
-        CB16 ? A.w_guard[0] : 1.0f);
+        [&](int, int e, float xe, float& hi, float& lo) { exact_resid<true>(A, 1, it, ev[0] + e, xe, hi, lo); },
+        A.w_guard[0]);
 }
 
-template <bool CB16, bool GATED>
 __global__ void __launch_bounds__(kThreads, kEpilogueCtasPerSm) epilogue_kernel(const __grid_constant__ ExtrapArgs A) {
     constexpr long long TE = epilogue_tile_elems;
     after_previous();
@@ -88,25 +70,24 @@ __global__ void __launch_bounds__(kThreads, kEpilogueCtasPerSm) epilogue_kernel(
         const long long v0 = e0 + (long long)threadIdx.x * kVecElems;
         if (A.vec_ok[it] && v0 + kVecElems <= numel) {
             const long long ev[1] = {v0};
-            epilogue_vector<CB16, GATED>(A, it, ev);
+            epilogue_vector(A, it, ev);
         } else if (A.vec_ok[it]) {  // the end of the ragged last tile of an aligned item
-            for (long long e = v0; e < numel && e < v0 + kVecElems; ++e) scalar_element<CB16>(A, 1, it, e);
+            for (long long e = v0; e < numel && e < v0 + kVecElems; ++e) scalar_element<true>(A, 1, it, e);
         } else {  // misaligned item: element-wise, adjacent threads on adjacent elements
             const long long end = e0 + TE < numel ? e0 + TE : numel;
-            for (long long e = e0 + threadIdx.x; e < end; e += kThreads) scalar_element<CB16>(A, 1, it, e);
+            for (long long e = e0 + threadIdx.x; e < end; e += kThreads) scalar_element<true>(A, 1, it, e);
         }
     }
 }
 
 }  // namespace
 
-// Only the case the host runs here is instantiated: bf16 features, no gates.
 cudaError_t launch_epilogue(const ExtrapArgs& a, int grid, cudaStream_t s) {
-    return launch_overlapped(epilogue_kernel<true, false>, grid, kThreads, 0, s, a);
+    return launch_overlapped(epilogue_kernel, grid, kThreads, 0, s, a);
 }
 
 cudaError_t epilogue_blocks_per_sm(int* blocks) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, epilogue_kernel<true, false>, kThreads, 0);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, epilogue_kernel, kThreads, 0);
 }
 
 }  // namespace cbk
