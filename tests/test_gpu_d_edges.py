@@ -322,3 +322,61 @@ def test_wide_gate_rows(cb, H, K, cache, io, members, hidden):
     so, sr, _ = walk.expected_and_compare(target, outs, resid, rh, out_dtype=io, resid_dtype=io, G=G)
     assert so["bad"] == 0 and sr["bad"] == 0, (so, sr)
     walk.close()
+
+
+@pytest.mark.parametrize("entry", ["step", "noalloc"])
+@pytest.mark.parametrize("small", [True, False])
+def test_overlapping_launches_of_mixed_plans(cb, H, entry, small):
+    """Steps in a row whose buffers lie partly off the 16-byte grid (two launches
+    each) on hidden states that each leaves to the next, full steps with hidden
+    states between them, and the status handover's own launch after each: bit for
+    bit what the same calls give when every one is waited for."""
+    shape = (1, 77, 136) if small else (2, 256, 1152)
+    tensors = [workloads.TensorSpec(g, b, shape, g) for g in range(6) for b in range(2)]
+    w = workloads.Workload(name="mixed", tensors=tensors, K=4, cache_dtype="bf16", T=0, r=0, t_min=0.0, t_max=999.0,
+                           timesteps=[], degree=6, noise=0.1, seed=43)
+    nodes = [900.0 - 40.0 * k for k in range(10)]
+    got = {}
+    for wait in (True, False):
+        walk = H.Walk(w, node_t=nodes)
+        feats = [[workloads.trajectory(w, i, t, k, "cuda") for i in range(len(tensors))] for k, t in enumerate(nodes)]
+        resid = [_shifted(shape, torch.bfloat16, g % 2)[0] for g in range(6)]
+        for g, x in enumerate(resid):
+            x.copy_(workloads.hidden_state(w, g, "cuda"))
+        outs = [_shifted(shape, torch.bfloat16, (i // 2) % 2)[0] for i in range(len(tensors))]
+        status = torch.full((24,), -1, dtype=torch.int32).pin_memory()
+        torch.cuda.synchronize()
+        n = 0
+
+        def done():
+            if wait:
+                torch.cuda.synchronize()
+
+        for k in range(4):
+            cb.cb_cache_push(walk.plan, feats[k], cb.CB_BF16, nodes[k])
+            done()
+        for k in range(4, 10):
+            for i in range(4):
+                t = nodes[k - 1] - 5.0 * (i + 1)
+                if entry == "step":
+                    cb.cb_extrapolate(walk.plan, t, outs, cb.CB_BF16, resid, cb.CB_BF16)
+                    status[n] = 0
+                else:
+                    slot_t, head, _ = cb.cb_plan_history(walk.plan, 4)
+                    cb.cb_extrapolate_noalloc(walk.plan, walk.cache, walk.cache.numel() - cb.CB_STATUS_BYTES, slot_t, head,
+                                              t, outs, cb.CB_BF16, resid, cb.CB_BF16, status=status[n:])
+                n += 1
+                done()
+            cb.cb_cache_push_residual(walk.plan, outs if k % 2 else feats[k], cb.CB_BF16, nodes[k], resid, cb.CB_BF16)
+            done()
+        torch.cuda.synchronize()
+        assert cb.cb_plan_device_status(walk.plan) == 0 and not status.any()
+        got[wait] = [x.view(torch.int16).clone() for x in outs + resid]
+        got[wait].append(walk.cache[: walk.cache.numel() - cb.CB_STATUS_BYTES].clone())
+        walk.close()
+    assert all(torch.equal(a, b) for a, b in zip(got[True][:-1], got[False][:-1]))
+    offs, slot = H.slot_layout([s.numel for s in tensors], 2)
+    for j in range(4):  # the slots, but for their padding
+        for i, s in enumerate(tensors):
+            lo = j * slot + offs[i]
+            assert torch.equal(got[True][-1][lo:lo + 2 * s.numel], got[False][-1][lo:lo + 2 * s.numel])
