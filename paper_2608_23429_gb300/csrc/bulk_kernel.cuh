@@ -280,9 +280,10 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
     void* resid = GROUPED ? A.resid[it] : nullptr;
     // Gates come with the stage (staged_gates), else from global memory, asked
     // for before the wait, and wait in registers through the sums; with bf16
-    // sources and K >= 7 the sums need those (DiT-XL/2 512^2, K = 8: 763 against
-    // 779 us; K = 6: 671 against 645, K = 4: 536 against 528).
-    constexpr bool LATE_GATES = GATED && !RAGGED && CB16 && K >= 7;
+    // sources and K >= 5 the sums need those, and the gates are read after them
+    // (DiT-XL/2 512^2, fp32 gates, before -> after the sums: K = 4 528 -> 536 us, K = 5
+    // 615 -> 600, K = 6 663 -> 646, K = 7 727 -> 711, K = 8 812 -> 780).
+    constexpr bool LATE_GATES = GATED && !RAGGED && CB16 && K >= 5;
     constexpr bool STAGED_GATES = GATED && !RAGGED && staged_gates(K, CB16);
     const int held = RAGGED && !FULL ? (int)ragged_bytes<ES>(A, n) / ES : Sh::tile;  // elements in the chunks
     auto in = [&](int i) { return FULL || i < n; };
@@ -415,7 +416,7 @@ __device__ __forceinline__ bool precise_tile(const ExtrapArgs& A, int it, long l
                 want = false;
             }
         }
-        member_precise<K, CB16, U, GATED, GROUPED>(
+        member_precise<K, CB16, U, GATED>(
             A, want, raw, resid != nullptr, acc, fin,
             [&](int v, float (&gv)[8]) {
                 if constexpr (GATED) {

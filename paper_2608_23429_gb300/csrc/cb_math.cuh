@@ -706,13 +706,11 @@ struct Finite {
 // The output type and what is wanted are asked once per vector, not per pair:
 // branches between the pairs kept their chains from overlapping and held 10 to
 // 30 registers more (gated fp32 hidden states, DiT-XL/2 512^2: K = 2 520 -> 430 us,
-// K = 4 585 -> 528, K = 8 798 -> 765; the off-grid gated step of 24 x [3, 333, 577]
-// 54 -> 48; a full step of DiT-XL/2 256^2 with fp32 hidden states and gates 230 -> 198).
-// Predictions alone (!GROUPED) with K = 5, 6 and 8, which HBM bounds, stream
-// better with a branch per pair, which spreads the consumers' stores (K = 8
-// 738 against 752 us, K = 6 585 against 608, K = 5 564 against 573; K = 7 704 against 670
-// and K = 4 504 against 496 the other way).
-template <int K, bool CB16, int UV, bool GATED, bool GROUPED, typename Gate, typename Put>
+// K = 4 585 -> 528; the off-grid gated step of 24 x [3, 333, 577] 54 -> 48; a full
+// step of DiT-XL/2 256^2 with fp32 hidden states and gates 230 -> 198). fp32
+// predictions alone, which HBM bounds, are as fast either way (K = 4..8 504, 564,
+// 606, 670, 735 -> 492, 570, 586, 670, 736 us).
+template <int K, bool CB16, int UV, bool GATED, typename Gate, typename Put>
 __device__ __forceinline__ void member_precise(const ExtrapArgs& A, bool want, const RawVecs<K, CB16, UV>& raw,
                                                bool accumulate, Acc<UV>& acc, Finite& fin, Gate gate, Put put) {
 #pragma unroll
@@ -724,27 +722,17 @@ __device__ __forceinline__ void member_precise(const ExtrapArgs& A, bool want, c
             if (accumulate) gate(u, g);
         if (want) {
             uint32_t o[8];
-            auto pair = [&](bool bf16, int q) {
-                float2 hi = add2(sv[q], cv[q]), lo = hi;
-                if (bf16) two_sum2(sv[q], cv[q], hi, lo);
-                put_pair(o, bf16, q, hi, lo);
-                if (K > 2) fin.see(hi);
-            };
             auto pairs = [&](bool bf16) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) pair(bf16, q);
+                for (int q = 0; q < 4; ++q) {
+                    float2 hi = add2(sv[q], cv[q]), lo = hi;
+                    if (bf16) two_sum2(sv[q], cv[q], hi, lo);
+                    put_pair(o, bf16, q, hi, lo);
+                    if (K > 2) fin.see(hi);
+                }
                 put(u, bf16, o);
             };
-            if constexpr (!GROUPED && K >= 5 && K != 7) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (A.out_bf16)
-                        pair(true, q);
-                    else
-                        pair(false, q);
-                }
-                put(u, A.out_bf16, o);
-            } else if (A.out_bf16) {
+            if (A.out_bf16) {
                 pairs(true);
             } else {
                 pairs(false);

@@ -55,7 +55,7 @@ __device__ __forceinline__ void precise_vectors(const ExtrapArgs& A, int it, con
         void* out = member_out<K, CB16, UV>(A, first + m, ev, raw);
         float g[UV][8];
         if constexpr (GATED) load_gates<UV>(A, first + m, gi, g);
-        member_precise<K, CB16, UV, GATED, true>(
+        member_precise<K, CB16, UV, GATED>(
             A, out != nullptr, raw, resid != nullptr, acc, fin,
             [&](int u, float (&gv)[8]) {
 #pragma unroll
