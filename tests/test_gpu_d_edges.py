@@ -380,3 +380,78 @@ def test_overlapping_launches_of_mixed_plans(cb, H, entry, small):
         for i, s in enumerate(tensors):
             lo = j * slot + offs[i]
             assert torch.equal(got[True][-1][lo:lo + 2 * s.numel], got[False][-1][lo:lo + 2 * s.numel])
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+def test_overlapping_launches_captured_across_streams(cb, H, shift):
+    """A captured fork and join: launches whose graph node follows a kernel, a copy,
+    another stream's kernel, or two streams' at once, each waiting for all of them.
+    Replays on new inputs give what the same calls give outside of a graph."""
+    tensors = [workloads.TensorSpec(g, b, (1, 200, 1152), g) for g in range(4) for b in range(2)]
+    w = workloads.Workload(name="fork", tensors=tensors, K=3, cache_dtype="bf16", T=0, r=0, t_min=0.0, t_max=999.0,
+                           timesteps=[], degree=6, noise=0.1, seed=47)
+    nodes = [900.0, 860.0, 820.0]
+    walks = [H.Walk(w, node_t=nodes) for _ in range(2)]
+    bf = torch.bfloat16
+    bufs = [[[_shifted(s.shape, bf, shift)[0] for s in tensors] for _ in range(2)] for _ in range(2)]  # outputs, inputs
+    resid = [[_shifted((1, 200, 1152), bf, shift if g % 2 else 0)[0] for g in range(4)] for _ in range(2)]
+    status = torch.full((2,), -1, dtype=torch.int32).pin_memory()
+    side = torch.cuda.Stream()
+
+    def fill(salt):
+        for k, walk in enumerate(walks):
+            cb.cb_plan_reset(walk.plan)
+            for j, t in enumerate(nodes):
+                cb.cb_cache_push(walk.plan, [workloads.trajectory(w, i, t, 10 * salt + 3 * k + j, "cuda") for i in range(8)],
+                                 cb.CB_BF16, t)
+            for g, x in enumerate(resid[k]):
+                x.copy_(workloads.hidden_state(w, g, "cuda", salt=10 * salt + k))
+            for x in bufs[0][k] + bufs[1][k]:
+                x.zero_()
+
+    def step():
+        here = torch.cuda.current_stream()
+        outs, ins = bufs
+        cb.cb_extrapolate(walks[0].plan, 800.0, outs[0], cb.CB_BF16, resid[0], cb.CB_BF16, stream=here)
+        side.wait_stream(here)
+        # on the side: after another stream's kernel; then after a copy
+        cb.cb_extrapolate(walks[1].plan, 800.0, outs[1], cb.CB_BF16, resid[0], cb.CB_BF16, stream=side)
+        with torch.cuda.stream(side):
+            for a, b in zip(ins[1], outs[1]):
+                a.copy_(b)
+        cb.cb_extrapolate(walks[1].plan, 790.0, ins[1], cb.CB_BF16, resid[1], cb.CB_BF16, stream=side)
+        cb.cb_extrapolate(walks[0].plan, 790.0, ins[0], cb.CB_BF16, stream=here)
+        here.wait_stream(side)
+        # after both streams' kernels
+        slot_t, head, _ = cb.cb_plan_history(walks[0].plan, 3)
+        cb.cb_extrapolate_noalloc(walks[0].plan, walks[0].cache, walks[0].cache.numel() - cb.CB_STATUS_BYTES, slot_t, head,
+                                  780.0, outs[0], cb.CB_BF16, resid[1], cb.CB_BF16, status=status, stream=here)
+        for a, b in zip(outs[1], outs[0]):
+            a.add_(b)
+
+    def result():
+        torch.cuda.synchronize()
+        assert int(status[0]) == 0 and all(cb.cb_plan_device_status(x.plan) == 0 for x in walks)
+        return [x.view(torch.int16).clone() for pair in bufs + [resid] for xs in pair for x in xs]
+
+    main = torch.cuda.Stream()
+    want = []
+    for salt in (0, 1):
+        fill(salt)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(main):
+            step()
+        want.append(result())
+    fill(0)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=main):
+        step()
+    for salt in (0, 1, 0):
+        fill(salt)
+        status.fill_(-1)
+        torch.cuda.synchronize()
+        graph.replay()
+        assert all(torch.equal(a, b) for a, b in zip(result(), want[salt])), salt
+    for walk in walks:
+        walk.close()
