@@ -862,7 +862,7 @@ def main():
     ap.add_argument("--feat-dtype", default="bf16", choices=["bf16", "fp32"],
                     help="type of the full step's features (--step full / full-fused)")
     ap.add_argument("--kernel", default="auto", choices=["auto", "direct", "bulk"],
-                    help="skipped-step kernel variant (both compute identical bits)")
+                    help="skipped-step kernel variant")
     ap.add_argument("--history", type=int, default=0,
                     help="history size K instead of the workload's own (1..8; changes the schedule's warm-up)")
     ap.add_argument("--scale", type=int, default=1,

@@ -207,9 +207,9 @@ int cb_extrapolate_ring(cb_plan* plan, const double* slot_t, int head, double t_
  *       as cb_extrapolate_ring. Every slot must hold an entry.
  * status: host pointer (may be NULL). It receives the launch's device status
  *       word (CB_DEV_* codes, 0 = none) once the stream has reached the end
- *       of this call. The device writes it when *status is pinned memory.
- *       With ordinary memory it is copied, and this call waits for the launch
- *       to finish.
+ *       of this call. The device writes it when *status is pinned memory on a
+ *       4-byte boundary. Otherwise it is copied, and with ordinary memory this
+ *       call waits for the launch to finish.
  *
  * Allocation: the call allocates no device memory and no pinned host memory.
  * Its status block is a file-scope device array of CB_STATUS_BYTES (256) bytes. Every GPU that
@@ -227,7 +227,8 @@ int cb_extrapolate_ring(cb_plan* plan, const double* slot_t, int head, double t_
  * or read another's code. Their outputs are unaffected.
  * Errors: as cb_extrapolate_ring (CB_ERR_UNBOUND excepted), plus CB_ERR_ALIGN
  * for hist and CB_ERR_CUDA when the status block cannot be reached. A
- * CB_ERR_CUDA from the status read-back comes after the launch was enqueued. */
+ * CB_ERR_CUDA from the status read-back comes after the launch was enqueued;
+ * what that launch records is cleared by the next call that asks, not told to it. */
 int cb_extrapolate_noalloc(cb_plan* plan, const void* hist, size_t hist_bytes, const double* slot_t,
                            int head, double t_target, void* const* outs, cb_dtype out_dtype,
                            void* const* resid, cb_dtype resid_dtype, int* status, void* stream);
@@ -310,7 +311,12 @@ int cb_plan_history(const cb_plan* plan, double* slot_t, int* head, int* count);
  * kernel: the direct-load kernel (each thread loads its K vectors from HBM) or
  * the bulk-copy pipeline (a producer warp stages the K chunks of each tile in
  * shared memory with cp.async.bulk; a persistent grid of one or two CTAs per
- * SM); both compute identical bits. CB_OPT_WAIT_NS bounds every wait of the bulk kernel
+ * SM). Both meet the accuracy stated at cb_extrapolate. They give identical
+ * bits for finite values in a tensor's whole tiles (of at most 4864 elements) in
+ * buffers on the 16-byte grid, where a group's members fit the pipeline together or
+ * results are fp32. Elsewhere (the end of a tensor, other buffers, larger groups)
+ * they sum in different ways, and a bf16 result may differ by one ulp.
+ * CB_OPT_WAIT_NS bounds every wait of the bulk kernel
  * on a shared-memory barrier; a wait that runs out makes the kernel record a
  * CB_DEV_* code in the device status word and return early (its outputs are
  * then incomplete). Errors: CB_ERR_ARG. */

@@ -1,7 +1,9 @@
-// Skipped-step kernel, bulk-copy pipeline variant (same arithmetic and bits as
-// the direct kernel on whole tiles; a tensor's ragged last tile takes the
-// compensated path for every element here. Sec. 3.3, Eq. for f_t; Alg. 1,
-// extrapolation branch).
+// Skipped-step kernel, bulk-copy pipeline variant (Sec. 3.3, Eq. for f_t; Alg. 1,
+// extrapolation branch). It gives the direct kernel's bits, for finite values, in
+// the whole tiles of items on the 16-byte grid, where the launch holds its groups
+// or has fp32 results. The compensated sums take the place of the direct kernel's
+// guarded ones in ragged last tiles and in bf16 groups too large to hold, and of
+// its element-wise Dot2 for items off the grid.
 //
 // One or two CTAs per SM (see Shape). A producer lane moves, for every work unit
 // (one tile of one branch tensor), the K history chunks of the tile (8 KB each,

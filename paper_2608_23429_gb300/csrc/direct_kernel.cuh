@@ -11,7 +11,8 @@
 //     8-element vectors, fp32: one) before any arithmetic;
 //   * the weights arrive as kernel parameters (fp32 high/low pairs).
 // The arithmetic is in cb_math.cuh. The bulk-copy pipeline variant
-// (bulk_kernel.cuh) computes the same bits from shared memory. GATED: the
+// (bulk_kernel.cuh) computes from shared memory; its head says where it gives the
+// same bits. GATED: the
 // hidden states receive g_b * P_b (per-(batch, channel) gates); instantiated
 // in extrapolate_gated.cu, the un-gated kernels in extrapolate.cu, those with
 // fp32 predictions or hidden states in extrapolate_precise.cu.

@@ -13,8 +13,8 @@
 // before any arithmetic), then storing the slot vectors and the new hidden
 // state. The arithmetic is the skipped-step kernels' (cb_math.cuh), with the
 // same choices per case as the direct-load kernel, so the kernels write
-// identical bits (the bulk kernel's ragged last tiles, computed by the
-// compensated path throughout, aside).
+// identical bits (the bulk kernel's ragged last tiles and items off the 16-byte
+// grid, which take the compensated path throughout, aside).
 //
 // Each thread has (members + 1) loads in flight, so the kernel streams well
 // only when groups are large: the host runs it for ungated bf16 features and
