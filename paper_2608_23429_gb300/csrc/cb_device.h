@@ -142,7 +142,8 @@ constexpr int kMaxStages = 16;
 // for fp32 ones (with the producer a multiple of the four schedulers). GB300,
 // DiT-XL/2 512^2, K = 4, fp32 hidden states, with and without gates: 7 warps
 // 1048 us, 11 871 / 666 us, 15 607 / 509 us, 19 577 / 458 us, 23 (spilling)
-// 746 / 512 us; 11 against 15 warps for fp32 sources, K = 8: 379 / 454 us.
+// 746 / 512 us, at a time when the consumers branched once per pair (19 warps take
+// 528 / 443 us now); 11 against 15 warps for fp32 sources, K = 8: 379 / 454 us.
 //
 // Others: two CTAs of 8 consumer warps, else one (16 for bf16 tiles): two
 // for K = 1, for bf16 prediction-only launches (not `grouped`) with
@@ -159,10 +160,10 @@ struct BulkShape {
 };
 // Compensated launches whose gate rows are staged with their member: where the
 // loads' latency counts more than the rows' room and traffic (GB300, 28 groups of
-// two, [8, 256, 1152]: fp32 sources, K = 1 and 2 343 -> 268 and 380 -> 313 us,
-// K = 4 481 -> 460 us; bf16 sources and gates, K = 1 and 2 240 -> 226 and 305 ->
-// 289 us, but with fp32 gates 280 -> 287 us for K = 2 and 586 -> 633 us for K = 4,
-// [4, 1024, 1152]).
+// two, [8, 256, 1152], gates from global memory -> staged: fp32 sources, K = 1, 2, 4,
+// 8 247 -> 207, 288 -> 247, 382 -> 381, 670 -> 670 us; bf16 sources, K = 1..4, bf16 gates
+// 204 -> 186, 228 -> 219, 251 -> 244, 280 -> 272 us, fp32 gates 185 -> 186, 217 -> 219,
+// 240 -> 245, 272 -> 276 us).
 __host__ __device__ constexpr bool staged_gates(int K, bool src_bf16) { return !src_bf16 || K <= 2; }
 __host__ __device__ constexpr BulkShape bulk_shape(int K, bool src_bf16, bool grouped, bool gated, bool precise,
                                                    bool strided) {

@@ -497,13 +497,13 @@ int launch_bulk(Launch& L, cbk::ExtrapArgs& A, bool strided) {
     }
     if (rc != CB_OK) return rc;
     if (A.stages < min_stages) {  // too deep for shared memory
-        // A group too large to hold: the compensated kernels hold none (GB300,
-        // 10 groups of 4 x [8, 256, 1152], K = 8: 290 us against 318 us for the
-        // direct-load kernel, 329 against 458 us with gates; 14 groups, K = 6: 310
-        // against 331 us; fp32 sources, 5 groups of 4 x [4, 256, 1152], K = 6..8:
-        // 102, 112, 125 against 109, 129, 139 us). bf16 sources with gates and
-        // K <= 6 are faster there (28 groups of 4 x [8, 256, 1152], K = 5 and 6:
-        // 578 and 705 against 684 and 757 us).
+        // A group too large to hold: the compensated kernels hold none (GB300, hidden
+        // states in bf16, 10 groups of 4 x [8, 256, 1152], K = 5..8: 162, 185, 219, 228 us
+        // against 175, 208, 247, 288 for the direct-load kernel, with gates K = 7 and 8
+        // 242 and 264 against 275 and 316; fp32 sources, 5 groups of 4 x [4, 256, 1152],
+        // K = 6 and 8: 85 and 108 against 94 and 135). bf16 sources with gates and
+        // K <= 6 are faster there (28 groups of 4 x [8, 256, 1152], K = 5 and 6: 484 and
+        // 571 against 553 and 608 us).
         if (!hold || (cb16 && K <= 6 && gated)) return launch_direct(L, A);
         A.precise = 1;
         return launch_bulk(L, A, false);
